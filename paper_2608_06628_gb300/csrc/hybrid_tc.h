@@ -47,6 +47,11 @@ cudaError_t launch_prefill(const hybrid_cfg &c, const void *K, const void *V, in
 cudaError_t launch_commit_red(const hybrid_cfg &c, const void *K, const void *V, int n_tok, const void *W,
                               void *const *states, int n_req, unsigned *err, cudaStream_t st);
 
+// Feature map of bf16 rows on the tensor cores (hybrid_phi.cu), F >= 64.
+bool phi_tc_supported(hybrid_dtype dt, long long n_rows, int group, int d, int F);
+cudaError_t launch_phi_tc(const void *X, int n_rows, int nh, int Hkv, int d, int F, const void *W, float *Phi,
+                          unsigned *err, cudaStream_t st);
+
 // Ragged prompts: request r folds tokens [tok[r], tok[r + 1]) of the packed K, V
 // [tok[n_req]][Hkv][d]; tok is a host array read at launch (its values travel in
 // the kernel parameters), so at most kMaxRaggedRequests requests per launch.

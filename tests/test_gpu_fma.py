@@ -1,5 +1,5 @@
-"""The CUDA-core kernels (float32 throughout) at the edges of their tiles, against the
-fp64 oracle: one row, one token, remainders of the 16 / 32 / 64-row tiles and of the
+"""The CUDA-core kernels (float32 throughout) and the feature map (tensor cores for bf16
+rows) at the edges of their tiles, against the fp64 oracle: one row, one token, remainders of the 16 / 32 / 64-row tiles and of the
 32-token chunks, every F, both head sizes, and batches that take each row-tile size.
 """
 import math
@@ -63,7 +63,9 @@ def test_step_and_commit(dt, n, Hq, Hkv, d, F, B):
 
 @pytest.mark.parametrize("dt", [F32, BF16])
 @pytest.mark.parametrize("d,F,nh,Hkv,n_rows", [(64, 16, 1, 1, 1), (128, 32, 6, 2, 17), (64, 64, 8, 4, 700),
-                                               (128, 128, 16, 4, 1237), (128, 256, 4, 4, 301), (64, 256, 2, 1, 65)])
+                                               (128, 128, 16, 4, 1237), (128, 256, 4, 4, 301), (64, 256, 2, 1, 65),
+                                               # several tensor-core tiles per CTA, W changing on the way
+                                               (64, 256, 8, 4, 5000), (128, 64, 2, 2, 40000), (128, 128, 24, 2, 50)])
 def test_feature_map(dt, d, F, nh, Hkv, n_rows):
     g = torch.Generator(device="cuda").manual_seed(d + F + n_rows)
     X = torch.randn((n_rows, nh, d), generator=g, device="cuda").to(dt)
