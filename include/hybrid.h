@@ -62,8 +62,10 @@
  * float32 or bfloat16.  The state is always float32.  Arithmetic is float32
  * throughout.  With bfloat16 inputs and F >= 64 the contractions of the
  * step (B a multiple of 16, G * B <= 128) and of the commit run on the
- * tensor cores (bf16 and tf32 operands, float32 accumulation); other shapes
- * and float32 inputs run float32 FMA kernels.
+ * tensor cores (bf16 and tf32 operands, float32 accumulation).  The step's
+ * other bfloat16 shapes run there too when G divides 128, with every float32
+ * operand as a sum of tf32 or bf16 parts (float32 accuracy); the rest and
+ * float32 inputs run float32 FMA kernels.
  *
  * Errors: argument checks run synchronously on the host and return
  * HYBRID_ERR_INVALID_ARG (null or misaligned pointer, inconsistent sizes) or

@@ -1,5 +1,6 @@
 // attn_fma.cuh -- the block-hybrid step of Section 3.1 on the CUDA cores, float32
-// throughout: every shape and dtype that the tensor-core kernels do not take.
+// throughout: float32 I/O, and the few bf16 shapes that the tensor-core kernels do not take
+// (G not a divisor of 128).
 //
 // One CTA takes RT of the G B query rows (row t G + h) of a unit (request, state head),
 // so that W, K, V and the state are read once per RT rows rather than once per query
@@ -10,15 +11,14 @@
 // What bounds it: the shared-memory and FMA pipes (a row costs 2 d F + 4 F d + 4 B d
 // operations; tensor cores cannot be used for float32 inputs without losing precision).
 // One request, 2 heads, d = F = 64, B = 16, float32: 26.6 us with one CTA per query head and
-// 16 rows, 8.8 us now; 32 requests, 16 : 4 heads, d = F = 128, B = 64, bf16, with the commit:
-// 695 us, 220 us now.
+// 16 rows, 8.8 us now (the host's launch time is 8 us).
 #pragma once
 
 #include <atomic>
 
 #include "fma_tile.cuh"
 #include "hybrid_kernels.h"
-#include "tc_ptx.cuh"
+#include "tc_pipeline.cuh"
 
 namespace hyb {
 namespace fma {
@@ -282,7 +282,9 @@ cudaError_t launch_opted(Kern kern, std::atomic<unsigned long long> &opted, unsi
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3(grid);
     lc.blockDim = dim3(kThreads);
-    lc.dynamicSmemBytes = smem;
+    // up to a CTA per SM: ask for the SM's shared memory, or the block scheduler puts two on
+    // one SM while others idle
+    lc.dynamicSmemBytes = cluster == 1 && grid <= (unsigned)pipe::sm_count() && smem < 118 * 1024 ? 118 * 1024 : smem;
     lc.stream = st;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

@@ -9,7 +9,6 @@
 #include <cooperative_groups.h>
 
 #include "attn_fma.cuh"
-#include "tc_pipeline.cuh"
 
 namespace hyb {
 

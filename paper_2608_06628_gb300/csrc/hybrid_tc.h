@@ -20,6 +20,13 @@ cudaError_t launch_attn_tc(const hybrid_cfg &c, const void *Q, const void *K, co
                            const void *W, const float *alpha, void *const *states, int n_req,
                            void *O, unsigned *err, cudaStream_t st);
 
+// Step of the other bf16 shapes at float32 accuracy, operands split into tf32 and bf16
+// parts (hybrid_attn_split.cu); needs G to divide 128.
+bool attn_split_supported(const hybrid_cfg &c);
+cudaError_t launch_attn_split(const hybrid_cfg &c, const void *Q, const void *K, const void *V, const void *W,
+                              const float *alpha, void *const *states, int n_req, void *O, unsigned *err,
+                              cudaStream_t st);
+
 // Persistent step kernel, one unit at a time with both feature halves read out
 // at once (hybrid_step.cu).
 bool step_supported(const hybrid_cfg &c);

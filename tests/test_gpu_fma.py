@@ -39,10 +39,18 @@ SHAPES = [
     (F32, 38, 4, 4, 128, 128, 64),      # 64-row tiles
     (F32, 76, 2, 2, 64, 64, 64),
     (F32, 80, 4, 2, 128, 256, 24),
-    (BF16, 2, 4, 1, 128, 128, 64),      # 256 query rows to a state
+    (BF16, 2, 6, 2, 128, 128, 48),      # G = 3: no tensor-core step
+    (BF16, 1, 3, 1, 64, 32, 20),
+    # split operands on the tensor cores: items of 128 rows, the last one partial, one row,
+    # F < 64, more items than SMs
+    (BF16, 2, 4, 1, 128, 128, 64),
     (BF16, 3, 2, 2, 128, 64, 24),
     (BF16, 40, 8, 2, 64, 32, 48),
     (BF16, 2, 8, 1, 64, 256, 40),
+    (BF16, 1, 1, 1, 64, 16, 1),
+    (BF16, 2, 2, 2, 128, 16, 128),
+    (BF16, 1, 2, 1, 128, 256, 127),
+    (BF16, 45, 8, 4, 128, 128, 20),
 ]
 
 
@@ -59,6 +67,28 @@ def test_step_and_commit(dt, n, Hq, Hkv, d, F, B):
     S, z = pair.gpu_state()
     assert_parity(S, pair.S, dt, "state S", units="state")
     assert_parity(z, pair.z, dt, "state z", units="state")
+
+
+@pytest.mark.parametrize("F,k_scale", [(128, 1.0), (256, 8.0), (32, 24.0)])
+def test_split_step_limits(F, k_scale):
+    """Saturated gates, large scores, an empty prefix and a bad state pointer on the split step."""
+    wl = wk.Workload("split", BF16, 3, 8, 2, 128, F, 40, 62, k_scale=k_scale)
+    pair = Pair(wl)
+    pair.build_prefixes(np.array([80, 40, 40]))
+    Q, K, V = wk.block_qkv(wl, "split", pair.dev)
+    for a in (math.inf, -math.inf, 30.0, -30.0, 0.0):
+        alpha = torch.full((wl.Hq,), a, dtype=torch.float32, device=pair.dev)
+        got, want, _ = pair.step(Q, K, V, alpha)
+        assert_parity(got, want, BF16, f"alpha={a}", units="out")
+    ptrs = pair.ptrs.clone()
+    ptrs[1] = 0
+    O = torch.full_like(Q, 7.0)
+    H.hybrid_block_attn(pair.cfg, Q, K, V, pair.W, pair.alpha, ptrs, wl.n_req, O)
+    assert H.hybrid_check(check=False) == H.HYBRID_ERR_DEVICE
+    assert torch.all(O[1] == 7.0)
+    fresh = Pair(wl)
+    got, want, _ = fresh.step(Q, K, V)
+    assert_parity(got, want, BF16, "empty prefix", units="out")
 
 
 @pytest.mark.parametrize("dt", [F32, BF16])
