@@ -60,13 +60,6 @@ unsigned char *scratch()
     return p;
 }
 
-// ptrs[i] = base + i * stride (the state pointers of the scratch slots).
-__global__ void k_fill_ptrs(void **ptrs, unsigned char *base, size_t stride, int n)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) ptrs[i] = base + (size_t)i * stride;
-}
-
 bool aligned(const void *p, uintptr_t a) { return (reinterpret_cast<uintptr_t>(p) & (a - 1)) == 0; }
 
 hybrid_status check_cfg(const hybrid_cfg *c)
@@ -207,20 +200,11 @@ hybrid_status hybrid_block_attn_commit_logical(const hybrid_cfg *cfg, const void
     const size_t ptr_bytes = ((size_t)n_req * sizeof(void *) + 255) & ~(size_t)255;
     void **d_ptrs = reinterpret_cast<void **>(base);
     unsigned char *states = base + ptr_bytes;
-    {
-        // the launch's own status (not an error left over from earlier work)
-        size_t stride = sb;
-        int n = n_req;
-        void *args[] = {&d_ptrs, &states, &stride, &n};
-        const cudaError_t e = cudaLaunchKernel(reinterpret_cast<const void *>(&k_fill_ptrs),
-                                               dim3((unsigned)((n_req + 127) / 128)), dim3(128), args, 0, stream);
-        if (e != cudaSuccess) return HYBRID_ERR_CUDA;
-    }
-    s = hybrid_state_pack(cfg, S_logical, z_logical, d_ptrs, n_req, stream);
-    if (s != HYBRID_OK) return s;
+    if (hyb::launch_scratch_pack(*cfg, S_logical, z_logical, states, d_ptrs, n_req, stream) != cudaSuccess)
+        return HYBRID_ERR_CUDA;
     s = hybrid_block_attn_commit(cfg, Q, K, V, W, alpha, d_ptrs, n_req, O, stream);
     if (s != HYBRID_OK) return s;
-    return hybrid_state_unpack(cfg, d_ptrs, n_req, S_logical, z_logical, stream);
+    return from_cuda(hyb::launch_scratch_unpack(*cfg, states, n_req, S_logical, z_logical, stream));
 }
 
 // Commits of more tokens than this run the prefill kernel (measured crossover
