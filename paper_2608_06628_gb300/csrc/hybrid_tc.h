@@ -42,6 +42,12 @@ cudaError_t launch_fused(const hybrid_cfg &c, const void *Q, const void *K, cons
                          const float *alpha, void *const *states, int n_req, void *O, unsigned *err,
                          cudaStream_t st);
 
+// The same for F = 256, 32 columns of u at a time (hybrid_fused_wide.cu); G B <= 64.
+bool fused_wide_supported(const hybrid_cfg &c);
+cudaError_t launch_fused_wide(const hybrid_cfg &c, const void *Q, const void *K, const void *V, const void *W,
+                              const float *alpha, void *const *states, int n_req, void *O, unsigned *err,
+                              cudaStream_t st);
+
 // Commit / prefill as a reduction (hybrid_commit_red.cu): S += dS and z += dz are
 // added into the state in global memory by bulk reduce-adds; any n_tok >= 1.
 bool commit_red_supported(const hybrid_cfg &c);
