@@ -9,18 +9,23 @@
 // registers, with no exchange between threads.  dS^T = V^T phi(K)^T accumulates
 // in Tensor Memory over a run of chunks; dz is the token sum of phi(K), reduced
 // within each warp.  At the end of a run the increments are added into the
-// state in global memory by bulk reduce-adds (the float32 add happens at L2), so
-// runs of the same state may be split across CTAs.
+// state in global memory by reduce-adds (the float32 add happens at L2), so
+// runs of the same state may be split across CTAs.  Four warps of their own move
+// a run's dS^T out of Tensor Memory while the math warps go on with the next run:
+// 64 prompts of 1 to 4096 tokens, 4 heads, d = F = 128, went from 134 to 108 us
+// against the math warps staging the tiles in phi(K)'s place, which cost each run
+// 4.8 us on top of its 3.2 us a chunk and gave CTAs with several short runs up to
+// 148 us where others took 106.
 //
 // Work: the n_units * n_chunks chunks ((request, state head) units of T tokens,
 // 128-token chunks, the last one masked) are split into contiguous ranges, one
 // per CTA, so long prompts balance across SMs to within one chunk; a range
-// covers whole or partial units ("runs").  Warp roles (12 warps):
+// covers whole or partial units ("runs").  Warp roles (16 warps):
 //   warp 0      producer: W of each run, K and V of each chunk (TMA)
 //   warp 1      MMA issuer (one thread); owns the Tensor Memory allocation
-//   warp 2      storer: bulk reduce-adds of dz and the dS^T tiles
 //   warps 4-11  math: thread = (token 32*q4 + lane, half "part"); phi(K) rows
-//               into shared memory, dz; at the end of a run the dS^T tiles
+//               into shared memory, dz and its adds into z
+//   warps 12-15 drain: a run's dS^T tiles to shared memory and their bulk reduce-adds
 // Tensor Memory: U_k of two chunks at columns [0, F) and [F, 2F) (lanes =
 // tokens), dS^T at [256, 256 + 2F) (lanes = e, the index into d; phi+ features
 // first), formed by one N = 2F product per 16 tokens.
@@ -36,10 +41,10 @@ namespace {
 
 using namespace pipe;
 
-constexpr int kWarps = 12;
+constexpr int kWarps = 16;
 constexpr int kThreads = kWarps * 32;
 constexpr int kCT = 128;             // tokens per chunk (the M of U_k = K W)
-constexpr int kStage = 4;            // staging slots for dS^T tiles, inside the phi(K) buffer
+constexpr int kStage = 2;            // staging slots for dS^T tiles
 constexpr int kSmemLimit = 232448;
 constexpr int kOneCtaPerSm = 118 * 1024;
 constexpr uint32_t kColDS = 256;      // dS^T: phi+ features at [256, 256 + F), phi- at [256 + F, 256 + 2F)
@@ -51,7 +56,7 @@ struct PrefillArgs {
     void *const *states;
     unsigned *err;
     int n_units, T, Hkv, d, F, n_chunks;
-    uint32_t off_w, off_k, off_v, off_p, off_s, off_dz, off_bar;
+    uint32_t off_w, off_k, off_v, off_p, off_s, off_bar;
 };
 // Ragged prompts: request r owns tokens [tok[r], tok[r + 1]) of the packed K and V
 // and chunks [ch[r], ch[r + 1]) of each of its heads; carried in the parameters.
@@ -89,14 +94,12 @@ __device__ __forceinline__ int chunk_req(const PrefillRaggedArgs &a, long long c
 __device__ __forceinline__ long long req_chunk0(const PrefillRaggedArgs &a, int r) { return (long long)a.Hkv * a.ch[r]; }
 
 // Shared memory: [W: F/64 atoms of d rows][K: 2 atoms of 128 rows][V x 2: 2 atoms each]
-// [phi(K): 2F/64 atoms of 128 rows][dz: 4 x 2F][barriers].  K and V always have
+// [phi(K): 2F/64 atoms of 128 rows][dS^T: kStage slots of d rows x 128 B][barriers].  K and V always have
 // two atoms so that the M = 128 operand V^T stays inside the allocation for
 // d = 64 (its upper rows are never read back).  V is double-buffered so the next
-// chunk's V streams in while this chunk's dS^T runs.  At the end of a run the
-// phi(K) buffer, free once the run's last dS^T is done, stages the dS^T tiles
-// (kStage slots of d rows x 128 B).
+// chunk's V streams in while this chunk's dS^T runs.
 struct PLayout {
-    uint32_t off_w, off_k, off_v, off_p, off_s, off_dz, off_bar, bytes;
+    uint32_t off_w, off_k, off_v, off_p, off_s, off_bar, bytes;
 };
 
 PLayout make_playout(int d, int F)
@@ -107,8 +110,7 @@ PLayout make_playout(int d, int F)
     L.off_k = off; off += 2 * kAtom;
     L.off_v = off; off += 2 * 2 * kAtom;
     L.off_p = off; off += (uint32_t)(2 * F / 64) * kAtom;
-    L.off_s = L.off_p;
-    L.off_dz = off; off += (((uint32_t)4 * 2 * F * 4) + 1023) & ~1023u;
+    L.off_s = off; off += kStage * (uint32_t)d * 128;
     L.off_bar = off; off += 1024;
     L.bytes = off + 1024;
     if ((int)L.bytes < kOneCtaPerSm) L.bytes = kOneCtaPerSm;
@@ -193,8 +195,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_prefill(const __grid_constant__
     const int d = a.d, F = a.F;
     const int NCH = F / 32, NC = 2 * NCH;
     const uint32_t tile = (uint32_t)d * 128;
-    // staging slots that fit in the phi(K) buffer (2 for d = 128, F = 64)
-    const int NSS = min(kStage, (int)(((uint32_t)(2 * F / 64) * kAtom) / tile));
     const long long total = total_chunks(a);
     const long long lo = total * (long long)blockIdx.x / (long long)gridDim.x;
     const long long hi = total * (long long)(blockIdx.x + 1) / (long long)gridDim.x;
@@ -211,14 +211,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_prefill(const __grid_constant__
     uint64_t *pready = ukfree + 2;     // the chunk's phi(K) is written
     uint64_t *dsdone = pready + 1;     // the chunk's dS^T products are complete (phi(K) may be rewritten)
     uint64_t *segdone = dsdone + 1;    // the run's dS^T is complete
-    uint64_t *dsfree = segdone + 1;    // the math warps have read the run's dS^T
-    uint64_t *sfull = dsfree + 1;      // [kStage] a staging slot holds a dS^T tile
-    uint64_t *sempty = sfull + kStage;
-    uint64_t *dzready = sempty + kStage;
-    uint64_t *dzfree = dzready + 1;
-    uint64_t *sdrain = dzfree + 1;     // the run's staged tiles have been read (phi(K) may be rewritten)
-    uint64_t *mmadone = sdrain + 1;
-    const int n_bars = 20 + 2 * kStage;   // wfull .. mmadone
+    uint64_t *dsfree = segdone + 1;    // the drain warps have read the run's dS^T
+    uint64_t *mmadone = dsfree + 1;
+    const int n_bars = 17;             // wfull .. mmadone
     uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(bars + n_bars);
     volatile int *fail = reinterpret_cast<volatile int *>(tmem_holder + 1);
 
@@ -232,9 +227,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_prefill(const __grid_constant__
         mbar_init(pready, 8);
         mbar_init(&ukfree[0], 8);
         mbar_init(&ukfree[1], 8);
-        mbar_init(dsfree, 8);
-        mbar_init(dzready, 8);
-        for (int s = 0; s < kStage; ++s) mbar_init(&sfull[s], 4);   // the four warps of one part
+        mbar_init(dsfree, 4);
         *fail = 0;
         fence_mbar_init();
     }
@@ -248,7 +241,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_prefill(const __grid_constant__
     griddep_wait();
     const uint32_t tmem = *tmem_holder;
     uint8_t *stage = smem + a.off_s;
-    float *dzq = reinterpret_cast<float *>(smem + a.off_dz);   // [quarter][2F]
 
     if (warp == 0) {
         // ------------------------------------------------------------- producer
@@ -358,38 +350,48 @@ __global__ void __launch_bounds__(kThreads, 1) k_prefill(const __grid_constant__
             mma_commit(mmadone);
             mbar_wait(mmadone, 0, kWaitNs);
         }
-    } else if (warp == 2) {
-        // --------------------------------------------------------------- storer
-        if (lane == 0) {
-            uint32_t s = 0, sg = 0;
-            bool ok = true;
-            UnitCache uc;
-            for (ChunkWalk<A> w(a, lo, hi); w.more() && ok; w.next(a)) {
-                const ChunkPos p = w.pos(a);
-                float *Sg = uc.get(a, p.u);
-                if (!Sg || !p.last) continue;
-                // dz: the four quarters' token sums, each added into z
-                if (!wait_bar(dzready, s & 1u, fail)) break;
-                for (int q = 0; q < 4; ++q) {
-                    bulk_reduce_add_f32(Sg + (size_t)2 * F * d, dzq + q * 2 * F, 2 * F * 4);
-                    bulk_commit();
+    } else if (warp >= 12) {
+        // ------------------------------------------------------------ drain
+        // a run's dS^T out of Tensor Memory and into the state, beside the next run's chunks.
+        // A warp owns the 32 rows (e) of its lane quarter: 4 KB of each tile, staged in
+        // two slots of its own, so nothing here waits for another warp
+        const int e = 32 * (warp & 3) + lane;
+        const uint32_t lane_off = (uint32_t)(32 * (warp & 3)) << 16;
+        uint32_t s = 0;
+        UnitCache uc;
+        for (ChunkWalk<A> w(a, lo, hi); w.more(); w.next(a)) {
+            const ChunkPos p = w.pos(a);
+            float *Sg = uc.get(a, p.u);
+            if (!Sg || !p.last) continue;
+            if (__any_sync(0xffffffffu, !wait_bar(segdone, s & 1u, fail))) break;
+            tc_fence_after();
+            if (32 * (warp & 3) < d) {
+#pragma unroll 1
+                for (int t = 0; t < NC; ++t) {
+                    float v[32];
+                    tmem_ld32(tmem + kColDS + lane_off + 32 * t, v);
+                    tmem_wait_ld();
+                    if (lane == 0) bulk_wait_read_1();
+                    __syncwarp();
+                    uint8_t *rowp = stage + (size_t)(t & 1) * tile + e * 128;
+#pragma unroll
+                    for (int gq = 0; gq < 8; ++gq)
+                        *reinterpret_cast<float4 *>(rowp + ((gq ^ (e & 7)) << 4)) =
+                            make_float4(v[4 * gq], v[4 * gq + 1], v[4 * gq + 2], v[4 * gq + 3]);
+                    fence_proxy_async_smem();
+                    __syncwarp();
+                    if (lane == 0) {
+                        bulk_reduce_add_f32(Sg + (size_t)t * 32 * d + e * 32, rowp, 4096);
+                        bulk_commit();
+                    }
                 }
-                bulk_wait_read_all();
-                mbar_arrive(dzfree);
-                for (int t = 0; t < NC; ++t, ++sg) {
-                    const int slot = sg % NSS;
-                    if (!wait_bar(&sfull[slot], (sg / NSS) & 1u, fail)) { ok = false; break; }
-                    bulk_reduce_add_f32(Sg + (size_t)t * 32 * d, stage + (size_t)slot * tile, tile);
-                    bulk_commit();
-                    bulk_wait_read_all();
-                    mbar_arrive(&sempty[slot]);
-                }
-                if (!ok) break;
-                mbar_arrive(sdrain);
-                ++s;
             }
-            bulk_wait_all();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(dsfree);
+            ++s;
         }
+        if (lane == 0) bulk_wait_all();
     } else if (warp >= 4) {
         // ------------------------------------------------------------- math
         const int mt = tid - 128;
@@ -398,13 +400,14 @@ __global__ void __launch_bounds__(kThreads, 1) k_prefill(const __grid_constant__
         const uint32_t lane_off = (uint32_t)(32 * q4) << 16;
         const float sgn = part == 0 ? kLog2e : -kLog2e;
         uint8_t *pkb = smem + a.off_p;
-        uint32_t s = 0, i = 0, sg = 0;
+        uint32_t i = 0;
         float dzacc[4] = {0.f, 0.f, 0.f, 0.f};   // token sums of features part*F + 32*jj + lane
         bool ok = true;
         UnitCache uc;
         for (ChunkWalk<A> w(a, lo, hi); w.more() && ok; w.next(a)) {
             const ChunkPos p = w.pos(a);
-            if (!uc.get(a, p.u)) {
+            float *Sg = uc.get(a, p.u);
+            if (!Sg) {
                 if (mt == 0) raise_error(a.err, ERR_BAD_STATE_PTR);
                 continue;
             }
@@ -448,10 +451,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_prefill(const __grid_constant__
             // into the exponent's offset
             const float mo = m + __log2f(l);
             const bool full = 32 * q4 + 32 <= nt;   // warp-uniform: every token of the warp is valid
-            // phi(K) is rewritten once the previous chunk's dS^T has read it and, after
-            // a run's end, once the storer has read the tiles staged there
+            // phi(K) is rewritten once the previous chunk's dS^T has read it
             if (i > 0) bad = !wait_bar(dsdone, (i - 1) & 1u, fail) || bad;
-            if (p.first && s > 0) bad = !wait_bar(sdrain, (s - 1) & 1u, fail) || bad;
             if (active) {
 #pragma unroll 1
                 for (int jj = 0; jj < NCH; ++jj) {
@@ -505,56 +506,18 @@ __global__ void __launch_bounds__(kThreads, 1) k_prefill(const __grid_constant__
             }
             ++i;
             if (p.last) {
-                // dz of this run: each quarter's token sums, added into z by the storer
-                bad = (s > 0 && !wait_bar(dzfree, (s - 1) & 1u, fail)) || bad;
+                // dz of this run: each quarter's token sums, added into z
 #pragma unroll
                 for (int jj = 0; jj < 4; ++jj)
-                    if (jj < NCH) dzq[q4 * 2 * F + part * F + 32 * jj + lane] = dzacc[jj];
+                    if (jj < NCH && !bad) atomicAdd(Sg + (size_t)2 * F * d + part * F + 32 * jj + lane, dzacc[jj]);
                 dzacc[0] = dzacc[1] = dzacc[2] = dzacc[3] = 0.f;
-                fence_proxy_async_smem();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(dzready);
-                // the run's dS^T tiles into the staging ring, in the storer's order
-                bad = !wait_bar(segdone, s & 1u, fail) || bad;
-                tc_fence_after();
-                const int e = tok;
-#pragma unroll 1
-                for (int t = 0; t < NCH; ++t) {
-                    // tiles of this part: chunks part, part + 2 of each half
-                    const int h = t / (NCH / 2 > 0 ? NCH / 2 : 1);
-                    const int k = part + 2 * (t % (NCH / 2 > 0 ? NCH / 2 : 1));
-                    if (k >= NCH) continue;
-                    const int cidx = h * NCH + k;
-                    const uint32_t sgc = sg + cidx;
-                    const int slot = sgc % NSS;
-                    const bool okc = wait_bar(&sempty[slot], ((sgc / NSS) & 1u) ^ 1u, fail) && !bad;
-                    float v[32];
-                    tmem_ld32(tmem + kColDS + (uint32_t)(h * F) + lane_off + 32 * k, v);
-                    tmem_wait_ld();
-                    if (okc && e < d) {
-                        uint8_t *rowp = stage + (size_t)slot * tile + e * 128;
-#pragma unroll
-                        for (int gq = 0; gq < 8; ++gq)
-                            *reinterpret_cast<float4 *>(rowp + ((gq ^ (e & 7)) << 4)) =
-                                make_float4(v[4 * gq], v[4 * gq + 1], v[4 * gq + 2], v[4 * gq + 3]);
-                    }
-                    fence_proxy_async_smem();
-                    __syncwarp();
-                    if (lane == 0 && okc) mbar_arrive(&sfull[slot]);
-                    bad = bad || !okc;
-                }
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(dsfree);
-                sg += NC;
-                ++s;
             }
             if (__any_sync(0xffffffffu, bad) && *fail) ok = false;
         }
-        if (mt == 0 && *fail) raise_error(a.err, ERR_WAIT_TIMEOUT);
     }
 
     __syncthreads();
+    if (tid == 0 && *fail) raise_error(a.err, ERR_WAIT_TIMEOUT);
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc(tmem, 512);
@@ -601,7 +564,6 @@ bool fill_prefill_args(const hybrid_cfg &c, const void *K, const void *V, long l
     a.off_v = L.off_v;
     a.off_p = L.off_p;
     a.off_s = L.off_s;
-    a.off_dz = L.off_dz;
     a.off_bar = L.off_bar;
     return true;
 }
