@@ -17,6 +17,14 @@
 // 4.8 us on top of its 3.2 us a chunk and gave CTAs with several short runs up to
 // 148 us where others took 106.
 //
+// What bounds it: the math warps' latency, two warps per scheduler with about half of
+// the issue slots taken (2.7 us a chunk, 2.4 times its 64 KB at the memory's rate).
+// phi is formed on the 16x256b view of U_k: a thread holds four tokens of eight features,
+// so the token sum takes 24 adds and 7 shuffles per 32 x 32 values (31 shuffles and 62
+// selects on one token per thread) and a stmatrix stores four 8 x 8 blocks; 108 -> 95.7
+// us.  Two loads in flight per wait and four chains in the extremum: 92.0.  Sixteen math
+// warps in two groups of alternate chunks: 99.3 (80 registers, and phi(K) has one buffer).
+//
 // Work: the n_units * n_chunks chunks ((request, state head) units of T tokens,
 // 128-token chunks, the last one masked) are split into contiguous ranges, one
 // per CTA, so long prompts balance across SMs to within one chunk; a range
@@ -401,7 +409,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_prefill(const __grid_constant__
         const float sgn = part == 0 ? kLog2e : -kLog2e;
         uint8_t *pkb = smem + a.off_p;
         uint32_t i = 0;
-        float dzacc[4] = {0.f, 0.f, 0.f, 0.f};   // token sums of features part*F + 32*jj + lane
+        // token sums of features part*F + 32*jj + dzf
+        float dzacc[4] = {0.f, 0.f, 0.f, 0.f};
+        const int dzf = 8 * (lane >> 3) + 2 * (lane & 3) + ((lane >> 2) & 1);
+        const uint32_t p_w = smem_u32(pkb) + (uint32_t)(32 * q4 + (lane & 7)) * 128;
         bool ok = true;
         UnitCache uc;
         for (ChunkWalk<A> w(a, lo, hi); w.more() && ok; w.next(a)) {
@@ -413,38 +424,44 @@ __global__ void __launch_bounds__(kThreads, 1) k_prefill(const __grid_constant__
             }
             const int nt = p.nt;
             const bool active = 32 * q4 < nt;      // warp-uniform: the warp holds a valid token
-            const bool valid = tok < nt;
             const uint32_t ub = tmem + (i & 1) * F + lane_off;
             bool bad = !wait_bar(&ukready[i & 1], (i >> 1) & 1u, fail);
             tc_fence_after();
             // softmax of this token over its half: the extremum (max of u for phi+,
-            // min for phi-), then the sum of exponentials.  U stays unchanged in Tensor
+            // min for phi-), then the sum of exponentials in the features' order.  U stays unchanged in Tensor
             // Memory: the token's other half is computed from the same columns by a
             // thread of another warp
             float m = 0.f, l = 0.f;
             if (active) {
-                float ext = part == 0 ? -INFINITY : INFINITY;
+                // four chains, two loads in flight
+                float ex[4];
+#pragma unroll
+                for (int c = 0; c < 4; ++c) ex[c] = part == 0 ? -INFINITY : INFINITY;
 #pragma unroll 1
-                for (int jj = 0; jj < NCH; ++jj) {
-                    float x[32];
-                    tmem_ld32(ub + 32 * jj, x);
+                for (int jj = 0; jj < NCH; jj += 2) {
+                    float x[64];
+                    tmem_ld32(ub + 32 * jj, reinterpret_cast<float(&)[32]>(x[0]));
+                    tmem_ld32(ub + 32 * jj + 32, reinterpret_cast<float(&)[32]>(x[32]));
                     tmem_wait_ld();
                     if (part == 0) {
 #pragma unroll
-                        for (int t = 0; t < 32; ++t) ext = fmaxf(ext, x[t]);
+                        for (int t = 0; t < 64; ++t) ex[t & 3] = fmaxf(ex[t & 3], x[t]);
                     } else {
 #pragma unroll
-                        for (int t = 0; t < 32; ++t) ext = fminf(ext, x[t]);
+                        for (int t = 0; t < 64; ++t) ex[t & 3] = fminf(ex[t & 3], x[t]);
                     }
                 }
+                const float ext = part == 0 ? fmaxf(fmaxf(ex[0], ex[1]), fmaxf(ex[2], ex[3]))
+                                            : fminf(fminf(ex[0], ex[1]), fminf(ex[2], ex[3]));
                 m = ext * sgn;   // max of sgn * u (log2 units)
 #pragma unroll 1
-                for (int jj = 0; jj < NCH; ++jj) {
-                    float x[32];
-                    tmem_ld32(ub + 32 * jj, x);
+                for (int jj = 0; jj < NCH; jj += 2) {
+                    float x[64];
+                    tmem_ld32(ub + 32 * jj, reinterpret_cast<float(&)[32]>(x[0]));
+                    tmem_ld32(ub + 32 * jj + 32, reinterpret_cast<float(&)[32]>(x[32]));
                     tmem_wait_ld();
 #pragma unroll
-                    for (int t = 0; t < 32; ++t) l += ex2(fmaf(x[t], sgn, -m));
+                    for (int t = 0; t < 64; ++t) l += ex2(fmaf(x[t], sgn, -m));
                 }
             }
             // phi = 2^(sgn u - m) / l = 2^(sgn u - (m + log2 l)): the normaliser folds
@@ -454,35 +471,56 @@ __global__ void __launch_bounds__(kThreads, 1) k_prefill(const __grid_constant__
             // phi(K) is rewritten once the previous chunk's dS^T has read it
             if (i > 0) bad = !wait_bar(dsdone, (i - 1) & 1u, fail) || bad;
             if (active) {
-#pragma unroll 1
+                // offsets of this thread's four tokens (8 i + lane / 4)
+                float mt4[4];
+#pragma unroll
+                for (int i4 = 0; i4 < 4; ++i4) mt4[i4] = __shfl_sync(0xffffffffu, mo, 8 * i4 + (lane >> 2));
+#pragma unroll 2
                 for (int jj = 0; jj < NCH; ++jj) {
+                    // x[8 i + 2 j + h]: token 8 i + lane / 4, feature 8 j + 2 (lane mod 4) + h
                     float x[32];
-                    tmem_ld32(ub + 32 * jj, x);
+                    tmem_ld_16x256_x4(ub + 32 * jj, x);
+                    tmem_ld_16x256_x4(ub + 32 * jj + (16u << 16), x + 16);
                     tmem_wait_ld();
-                    if (full) {
 #pragma unroll
-                        for (int t = 0; t < 32; ++t) x[t] = ex2(fmaf(x[t], sgn, -mo));
-                    } else {
+                    for (int i4 = 0; i4 < 4; ++i4)
 #pragma unroll
-                        for (int t = 0; t < 32; ++t) x[t] = valid ? ex2(fmaf(x[t], sgn, -mo)) : 0.f;
+                        for (int c = 0; c < 8; ++c) x[8 * i4 + c] = ex2(fmaf(x[8 * i4 + c], sgn, -mt4[i4]));
+                    if (!full) {
+#pragma unroll
+                        for (int i4 = 0; i4 < 4; ++i4)
+                            if (32 * q4 + 8 * i4 + (lane >> 2) >= nt) {
+#pragma unroll
+                                for (int c = 0; c < 8; ++c) x[8 * i4 + c] = 0.f;
+                            }
                     }
-                    // row tok of the MN-major operand [token][feature], 64-feature atoms,
-                    // 16-byte granules permuted by (tok mod 8)
+                    // rows of the MN-major operand [token][feature], 64-feature atoms, 16-byte
+                    // granules permuted by (token mod 8): four 8 x 8 matrices per store, lane
+                    // 8 j + r addresses row r of granule j
                     const int f0 = part * F + 32 * jj;
-                    uint8_t *rowp = pkb + (f0 >> 6) * kAtom + tok * 128;
-                    const int g0 = (f0 & 63) >> 3;
+                    const uint32_t rowa = p_w + (uint32_t)(f0 >> 6) * kAtom + (((((f0 & 63) >> 3) + (lane >> 3)) ^ (lane & 7)) << 4);
 #pragma unroll
-                    for (int gq = 0; gq < 4; ++gq) {
-                        const uint4 w = make_uint4(pack_bf16x2(x[8 * gq], x[8 * gq + 1]), pack_bf16x2(x[8 * gq + 2], x[8 * gq + 3]),
-                                                   pack_bf16x2(x[8 * gq + 4], x[8 * gq + 5]), pack_bf16x2(x[8 * gq + 6], x[8 * gq + 7]));
-                        *reinterpret_cast<uint4 *>(rowp + (((g0 + gq) ^ (tok & 7)) << 4)) = w;
+                    for (int i4 = 0; i4 < 4; ++i4)
+                        stmatrix_x4(rowa + i4 * 1024, pack_bf16x2(x[8 * i4], x[8 * i4 + 1]), pack_bf16x2(x[8 * i4 + 2], x[8 * i4 + 3]),
+                                    pack_bf16x2(x[8 * i4 + 4], x[8 * i4 + 5]), pack_bf16x2(x[8 * i4 + 6], x[8 * i4 + 7]));
+                    // token sum over this warp's 32 tokens: four in the thread, then eight
+                    // lanes, each keeping one of the eight features
+                    float y[8];
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) y[c] = (x[c] + x[8 + c]) + (x[16 + c] + x[24 + c]);
+#pragma unroll
+                    for (int w2 = 4; w2 >= 1; w2 >>= 1) {
+                        const bool up = lane & (4 * w2);
+#pragma unroll
+                        for (int c = 0; c < w2; ++c) {
+                            const float send = up ? y[c] : y[c + w2];
+                            y[c] = (up ? y[c + w2] : y[c]) + __shfl_xor_sync(0xffffffffu, send, 4 * w2);
+                        }
                     }
-                    // token sum over this warp's 32 tokens: lane L gets feature f0 + L
-                    const float sum = warp_reduce32<0>(x, lane);
-                    if (jj == 0) dzacc[0] += sum;
-                    else if (jj == 1) dzacc[1] += sum;
-                    else if (jj == 2) dzacc[2] += sum;
-                    else dzacc[3] += sum;
+                    if (jj == 0) dzacc[0] += y[0];
+                    else if (jj == 1) dzacc[1] += y[0];
+                    else if (jj == 2) dzacc[2] += y[0];
+                    else dzacc[3] += y[0];
                 }
             } else {
                 // a warp beyond the chunk's tokens writes zero rows (the dS^T products
@@ -509,7 +547,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_prefill(const __grid_constant__
                 // dz of this run: each quarter's token sums, added into z
 #pragma unroll
                 for (int jj = 0; jj < 4; ++jj)
-                    if (jj < NCH && !bad) atomicAdd(Sg + (size_t)2 * F * d + part * F + 32 * jj + lane, dzacc[jj]);
+                    if (jj < NCH && !bad) atomicAdd(Sg + (size_t)2 * F * d + part * F + 32 * jj + dzf, dzacc[jj]);
                 dzacc[0] = dzacc[1] = dzacc[2] = dzacc[3] = 0.f;
             }
             if (__any_sync(0xffffffffu, bad) && *fail) ok = false;
