@@ -13,7 +13,8 @@
 // [R_m | r_m] = sum_{n > m} dR_n.  Through phi = [softmax(u), softmax(-u)],
 // u = x W:  du = p+ (g+ - <g+, p+>) - p- (g- - <g-, p->),  dW += x du^T.
 //
-// Kernels (128 threads; thread r owns row r of a tile and Tensor Memory lane r):
+// Kernels (128 threads, thread r owns row r of a tile and Tensor Memory lane r; k_phi_grad
+// has four threads per row):
 //   k_prefix_states one CTA per (sequence, state head, 32-feature slice): sweeps
 //                   the blocks in order with the slice of S^T accumulating in
 //                   Tensor Memory (S^T += V^T phi(K), bf16 MMA) and writes
@@ -22,15 +23,14 @@
 //                   feature-row image PT (S tiles: row f holds 32 consecutive e,
 //                   128-byte swizzle), whose d/32 tiles are K-major tf32
 //                   operands for S dN
-//   k_slot_scan     reverse exclusive running sums over the R slots of a
-//                   sequence (one CTA per (sequence, block, state head) below)
-//   k_phi_grad<Q>   query side: [U | scores] = Q [W | K^T], dO V^T, the merge
+//   k_slot_scan     reverse exclusive running sums over the R slots of a sequence
+//   k_phi_grad<Q>   query side (one CTA per sequence, block and state head): [U | scores] = Q [W | K^T], dO V^T, the merge
 //                   terms, dN into Tensor Memory, then S dN streamed over the PT
 //                   tiles; g . o = w g.sm_num/D + phi(q).(S dN) and the gate term
 //                   are formed from these fp32 products (the forward's rounded O is
 //                   not needed), then du_q and dR_n = phi(Q)^T [dN | dD];
-//                   key side: U = K W, V into Tensor Memory, R v + r over the
-//                   R tiles, du_k
+//                   key side (up to 128 keys of consecutive blocks per CTA): U = K W,
+//                   V into Tensor Memory, R v + r over the blocks' R tiles, du_k
 //   k_dw            dW_g = sum over query and key rows of x du^T, split over
 //                   row ranges; each CTA writes its partial sum
 //   k_grad_reduce   dW and d alpha from the per-CTA and per-block partial sums,
@@ -53,7 +53,8 @@ constexpr int kThreads = 128;
 constexpr int kSmemLimit = 232448;
 constexpr uint32_t kColS = 0, kColGv = 64, kColU = 256, kColY = 384, kColG = 0, kColDR = 0;
 constexpr int kDwStages = 3;   // shared-memory stages of k_dw
-constexpr int kGradThreads = 256;   // k_phi_grad: two threads (parts) per Tensor Memory lane
+constexpr int kGradThreads = 512;   // k_phi_grad: four threads (two parts x two subs) per Tensor Memory lane
+constexpr int kGradSlots = 3;       // k_phi_grad: ring slots of S / R tiles
 constexpr uint32_t kXchBytes = 14 * 1024;   // k_phi_grad: the parts' exchange of row partials
 
 struct TrainArgs {
@@ -94,14 +95,15 @@ __device__ __forceinline__ uint32_t swz(int r, int j)
 
 __device__ __forceinline__ void bulk_wait_read_1() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
 
-// Write 32 consecutive columns [c0, c0 + 32) of row r (values x, converted to
+// Write kN consecutive columns [c0, c0 + kN) of row r (values x, converted to
 // bf16) into a bf16 operand image with panel stride pstride.
-__device__ __forceinline__ void store_row32_bf16(uint8_t *img, uint32_t pstride, int r, int c0, const float (&x)[32])
+template <int kN>
+__device__ __forceinline__ void store_row_bf16(uint8_t *img, uint32_t pstride, int r, int c0, const float (&x)[kN])
 {
     uint8_t *base = img + (uint32_t)(c0 >> 6) * pstride;
     const int j0 = (c0 & 63) >> 3;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
+    for (int q = 0; q < kN / 8; ++q) {
         uint4 v;
         v.x = pack_bf16x2(x[8 * q + 0], x[8 * q + 1]);
         v.y = pack_bf16x2(x[8 * q + 2], x[8 * q + 3]);
@@ -141,31 +143,28 @@ __device__ __forceinline__ PhiStats phi_stats(uint32_t taddr, int F)
     return s;
 }
 
-// Partial statistics of the same over the 32-column chunks [j0, j1) only, to be
-// combined with the other chunks' by combine_stats.
-__device__ __forceinline__ PhiStats phi_stats_chunks(uint32_t taddr, int j0, int j1)
+// Partial statistics of one sign over the 32-column chunks [j0, j1) only, to be
+// combined with the other chunks' by combine_stats: max u and sum e^(u - max), or
+// min u and sum e^(min - u).
+template <bool kNeg>
+__device__ __forceinline__ void sign_stats_chunks(uint32_t taddr, int j0, int j1, float *out)
 {
-    PhiStats s{-INFINITY, 0.f, INFINITY, 0.f};
+    float m = kNeg ? INFINITY : -INFINITY, s = 0.f;
     float x[32];
     for (int j = j0; j < j1; ++j) {
         ptx::tmem_ld32(taddr + 32 * j, x);
         ptx::tmem_wait_ld();
 #pragma unroll
-        for (int k = 0; k < 32; ++k) {
-            s.mp = fmaxf(s.mp, x[k]);
-            s.mn = fminf(s.mn, x[k]);
-        }
+        for (int k = 0; k < 32; ++k) m = kNeg ? fminf(m, x[k]) : fmaxf(m, x[k]);
     }
     for (int j = j0; j < j1; ++j) {
         ptx::tmem_ld32(taddr + 32 * j, x);
         ptx::tmem_wait_ld();
 #pragma unroll
-        for (int k = 0; k < 32; ++k) {
-            s.sp += ex2((x[k] - s.mp) * kLog2e);
-            s.sn += ex2((s.mn - x[k]) * kLog2e);
-        }
+        for (int k = 0; k < 32; ++k) s += ex2((kNeg ? m - x[k] : x[k] - m) * kLog2e);
     }
-    return s;
+    out[0] = m;
+    out[1] = s;
 }
 // Statistics of the whole row from the two halves' (a first, then b: both threads
 // of a row combine in the same order and get the same bits).
@@ -201,7 +200,7 @@ RowLayout make_grad_layout(int d, int F, int B)
     uint32_t phase1 = Lr.off_v + kvbytes;
     Lr.ring_slot = (uint32_t)2 * F * 128;                            // 2F rows x 32 floats
     Lr.off_ring = 0;
-    const uint32_t ring = 2 * Lr.ring_slot;
+    const uint32_t ring = kGradSlots * Lr.ring_slot;
     off = phase1 > ring ? phase1 : ring;
     Lr.off_phi = off;                                               // 128 rows x 2F bf16; dO first
     off += (uint32_t)(2 * F / 64) * 128 * 128;
@@ -501,7 +500,16 @@ __global__ void k_slot_scan(float *buf0, float *buf1, int n_seq, int n_slots, si
 }
 
 // ---------------------------------------------------------------------------
-// k_phi_grad<kQuery>: one (sequence s, block n, state head g).
+// k_phi_grad<kQuery>: sequence s, state head g, block n (query side) or the 128 / B blocks
+// from n on (key side).  On the key side a block fills B of the 128 rows, so a CTA takes as
+// many blocks as fit: the row arithmetic is done once for all of them, each block's R tiles
+// multiply all rows, and the lanes of the other blocks are left out of that product's result.
+// What bounds it: the phases of a CTA follow one another (one CTA per SM: the operands and
+// tiles take its shared memory, a row's products its Tensor Memory), the key side also the
+// memory (its tiles, 128 KB per block and head, at 2.7 TB/s).  8 sequences x 1024 tokens,
+// 16:4 heads, d = F = 128: key side 91 us with a block per CTA -> 53 (four blocks of 32, a
+// ring of three tiles); query side 165 us with two threads per row -> 155 (four, dO from
+// its shared image, three tiles, R staged in the ring's slots).
 // ---------------------------------------------------------------------------
 template <bool kQuery>
 __global__ void __launch_bounds__(kGradThreads, 1) k_phi_grad(const __grid_constant__ TrainArgs a, RowLayout Lr)
@@ -510,32 +518,38 @@ __global__ void __launch_bounds__(kGradThreads, 1) k_phi_grad(const __grid_const
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = aligned_smem(smem_raw);
     const int tid = threadIdx.x, warp = tid >> 5;
-    // two threads per Tensor Memory lane (row): lr = the lane, part = which half of each
-    // row's columns the thread takes; warps w and w + 4 share lanes 32 (w & 3) ..
-    const int lr = tid & 127, part = tid >> 7;
+    // four threads per Tensor Memory lane (row): lr = the lane, part = which half of each
+    // row's columns, sub = the sign of the features where sums run over one sign, else a
+    // half of the part's columns; warps w, w + 4, .. share lanes 32 (w & 3) ..
+    const int lr = tid & 127, part = (tid >> 7) & 1, sub = tid >> 8;
     const int d = a.d, F = a.F, B = a.B, Hkv = a.Hkv, Hq = a.Hq, G = Hq / Hkv;
-    const int g = blockIdx.x % Hkv, n = (blockIdx.x / Hkv) % a.n_blk, s = blockIdx.x / (Hkv * a.n_blk);
+    // blocks [n, n + nb) of sequence s: one on the query side, up to 128 rows on the key side
+    const int nbk = kQuery ? 1 : 128 / B, n_grp = (a.n_blk + nbk - 1) / nbk;
+    const int g = blockIdx.x % Hkv, n = (blockIdx.x / Hkv) % n_grp * nbk, s = blockIdx.x / (Hkv * n_grp);
+    const int nb = min(nbk, a.n_blk - n);
     // Rows of the tile on Tensor Memory lanes: query side, lane r < G*B is token r / G,
-    // head r % G of the group (the order the TMA box lands in); key side, lane r < B is
-    // token r.  Lanes beyond are zero rows.
-    const int rows = kQuery ? G * B : B;
+    // head r % G of the group (the order the TMA box lands in); key side, lane r < nb * B is
+    // token r of the blocks.  Lanes beyond are zero rows.
+    const int rows = kQuery ? G * B : nb * B;
     const size_t hf = head_floats(d, F);
     const size_t t0 = (size_t)s * a.L + (size_t)n * B;
     const size_t kv_row = (size_t)Hkv * d;
     // tile source: PT slot n (query side: S_{n-1}) or R slot n (key side: R_n)
     const float *src = (kQuery ? a.PT : a.R) + (((size_t)s * a.n_blk + n) * Hkv + g) * hf;
+    const size_t src_blk = (size_t)Hkv * hf;   // to the next block's slot
 
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + Lr.off_bar);
     uint64_t *mbar = bars;          // MMA groups complete
-    uint64_t *full = bars + 1;      // [2] ring slot loaded
-    uint64_t *empty = bars + 3;     // [2] ring slot consumed
-    uint64_t *tbar = bars + 5;      // the phase-one operands have landed
-    uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(bars + 6);
+    uint64_t *full = bars + 1;      // [kGradSlots] ring slot loaded
+    uint64_t *empty = full + kGradSlots;    // [kGradSlots] ring slot consumed
+    uint64_t *tbar = empty + kGradSlots;    // the phase-one operands have landed
+    uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(tbar + 1);
     volatile int *fail = reinterpret_cast<volatile int *>(tmem_holder + 1);
     float *sRowDw = reinterpret_cast<float *>(tmem_holder + 2);  // [128] each query row's gate term
-    float *sZ = reinterpret_cast<float *>(smem + Lr.off_z);     // z_{n-1} or r_n
+    // z_{n-1}, or r of each block (2F floats a block, in the space of the query side's K and V)
+    float *sZ = reinterpret_cast<float *>(smem + (kQuery ? Lr.off_z : Lr.off_k));
     if (tid == 0) {
-        for (int i = 0; i < 6; ++i) mbar_init(&bars[i], 1);
+        for (int i = 0; i < 2 + 2 * kGradSlots; ++i) mbar_init(&bars[i], 1);
         *fail = 0;
         fence_mbar_init();
         prefetch_tensormap(&a.tmW);
@@ -561,15 +575,24 @@ __global__ void __launch_bounds__(kGradThreads, 1) k_phi_grad(const __grid_const
     griddep_wait();
 
     // ring of S / R tiles: in the phase-one operands' space on the query side (free once
-    // the first MMAs have run); the key side has phi's space to itself, so its first two
-    // tiles are loaded right away, next to the operands
+    // the first MMAs have run); the key side has phi's and [dN | dD]'s space to itself, so
+    // its first tiles are loaded right away, next to the operands.  Tile q is e-tile
+    // q mod (d / 32) of block q / (d / 32)
     const uint32_t ring_off = kQuery ? Lr.off_ring : Lr.off_phi;
+    const int NCHUNK = d / 32, n_tiles = nb * NCHUNK;
     int loads_issued = 0;
+    auto load_tile = [&](int q) {
+        const int slot = q % kGradSlots, b = q / NCHUNK;
+        mbar_arrive_expect_tx(&full[slot], Lr.ring_slot);
+        bulk_g2s(smem + ring_off + slot * Lr.ring_slot, src + b * src_blk + (size_t)(q - b * NCHUNK) * 64 * F,
+                 Lr.ring_slot, &full[slot]);
+        ++loads_issued;
+    };
     // phase one by TMA: [U | scores] = Q [W | K^T] and dO V^T (query side) or U = K W
     if (tid == 0) {
         const uint32_t qbytes = (uint32_t)(d / 64) * rows * 128, kvbytes = (uint32_t)(d / 64) * B * 128;
         const uint32_t wbytes = (uint32_t)(F / 64) * d * 128;
-        mbar_arrive_expect_tx(tbar, kQuery ? 2 * qbytes + 2 * kvbytes + wbytes : kvbytes + wbytes);
+        mbar_arrive_expect_tx(tbar, kQuery ? 2 * qbytes + 2 * kvbytes + wbytes : nb * kvbytes + wbytes);
         for (int p = 0; p < d / 64; ++p) {
             if (kQuery) {
                 tma_load_3d(smem + Lr.off_q + p * 128 * 128, &a.tmQ, 64 * p, g * G, (int)t0, tbar);
@@ -577,18 +600,24 @@ __global__ void __launch_bounds__(kGradThreads, 1) k_phi_grad(const __grid_const
                 tma_load_3d(smem + Lr.off_k + p * B * 128, &a.tmK, 64 * p, g, (int)t0, tbar);
                 tma_load_3d(smem + Lr.off_v + p * B * 128, &a.tmV, 64 * p, g, (int)t0, tbar);
             } else {
-                tma_load_3d(smem + Lr.off_q + p * 128 * 128, &a.tmK, 64 * p, g, (int)t0, tbar);
+                for (int b = 0; b < nb; ++b)
+                    tma_load_3d(smem + Lr.off_q + p * 128 * 128 + b * B * 128, &a.tmK, 64 * p, g, (int)t0 + b * B, tbar);
             }
         }
         for (int p = 0; p < F / 64; ++p) tma_load_2d(smem + Lr.off_w + p * d * 128, &a.tmW, 64 * p, g * d, tbar);
         if (!kQuery)
-            for (int c = 0; c < 2 && c < d / 32; ++c) {
-                mbar_arrive_expect_tx(&full[c], Lr.ring_slot);
-                bulk_g2s(smem + ring_off + c * Lr.ring_slot, src + (size_t)c * 64 * F, Lr.ring_slot, &full[c]);
-                ++loads_issued;
-            }
+            for (int q = 0; q < kGradSlots && q < n_tiles; ++q) load_tile(q);
     }
-    for (int f = tid; f < 2 * F; f += kGradThreads) sZ[f] = src[z_offset(f, d, F)];
+    for (int f = tid; f < nb * 2 * F; f += kGradThreads) sZ[f] = src[(f / (2 * F)) * src_blk + z_offset(f % (2 * F), d, F)];
+    // V rows of the key side: read here, used after the statistics
+    const bool valid = lr < rows;
+    uint4 graw[4];   // 32 columns of dO (query) or V (key): d = 64 leaves sub 1 without
+    const int ycol = part * (d / 2) + 32 * sub;
+    if (!kQuery) {
+        const uint4 *vrow = reinterpret_cast<const uint4 *>(a.V + (t0 + (valid ? lr : 0)) * kv_row + (size_t)g * d + ycol);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) graw[i] = valid && sub < d / 64 ? __ldg(vrow + i) : make_uint4(0, 0, 0, 0);
+    }
     bool ok = wait_bar(tbar, 0, fail);
     fence_proxy_async_smem();
     __syncthreads();
@@ -596,7 +625,6 @@ __global__ void __launch_bounds__(kGradThreads, 1) k_phi_grad(const __grid_const
     const uint32_t tmem = *tmem_holder;
     const uint32_t lane_off = (uint32_t)(warp & 3) * 32u << 16;
     const uint32_t tl = tmem + lane_off;
-    const int NCHUNK = d / 32;
     const uint32_t ring_u = smem_u32(smem + ring_off);
     if (tid == 0) {
         const uint32_t q_u = smem_u32(smem + Lr.off_q), w_u = smem_u32(smem + Lr.off_w);
@@ -618,26 +646,30 @@ __global__ void __launch_bounds__(kGradThreads, 1) k_phi_grad(const __grid_const
     }
     ok = wait_bar(mbar, 0, fail) && ok;
     tc_fence_after();
-    // query side: the phase-one operands are consumed, the first two tiles go into their space
-    if (kQuery && tid == 0 && ok) {
-        for (int c = 0; c < 2 && c < NCHUNK; ++c) {
-            mbar_arrive_expect_tx(&full[c], Lr.ring_slot);
-            bulk_g2s(smem + ring_off + c * Lr.ring_slot, src + (size_t)c * 64 * F, Lr.ring_slot, &full[c]);
-            ++loads_issued;
-        }
+    // query side: the phase-one operands are consumed, the first tiles go into their space
+    if (kQuery && tid == 0 && ok)
+        for (int q = 0; q < kGradSlots && q < n_tiles; ++q) load_tile(q);
+    // the thread's columns of dO, before phi(q) takes its space
+    if (kQuery) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            graw[i] = sub < d / 64 ? *reinterpret_cast<const uint4 *>(smem + Lr.off_do + (uint32_t)(ycol >> 6) * (128 * 128) +
+                                                                     swz(lr, ((ycol & 63) >> 3) + i))
+                                   : make_uint4(0, 0, 0, 0);
     }
 
-    // ---- row statistics: the two parts of a row each take half of its columns and
-    // exchange partial sums through shared memory (pair barrier of warps w, w + 4) ----
-    const bool valid = lr < rows;
+    // ---- row statistics: the four threads of a row each take one sign of half of its
+    // columns and exchange partial sums through shared memory (barrier of the warps that
+    // share the lanes).  Every sum keeps the order that two threads per row gave it ----
     const int hl = (kQuery && valid) ? lr % G : 0;                 // query head within the group
     const int tok = valid ? (kQuery ? lr / G : lr) : 0;            // token within the block
-    const size_t q_row = (size_t)Hq * d;
     const uint32_t pair_bar = 2 + (uint32_t)(warp & 3);
     float *x1 = reinterpret_cast<float *>(smem + Lr.off_x);        // [2][128][8] statistics
     float *x2 = x1 + 2 * 128 * 8;                                  // [2][128]    lin_den
     float *x3 = x2 + 2 * 128;                                      // [2][128][4] pass-0 dots
     const int uj0 = part * (F / 64), uj1 = uj0 + F / 64;           // this part's 32-column chunks of U
+    const int uc0 = part * (F / 2) + sub * (F / 4), np = F / 64;   // this thread's columns of U: np pieces of 16
+    const float *zr = kQuery ? sZ : sZ + tok / B * 2 * F;          // z or r of the row's block
     const float scale = rsqrtf((float)d);
     float w = 0.f;
     if (kQuery) {
@@ -646,10 +678,10 @@ __global__ void __launch_bounds__(kGradThreads, 1) k_phi_grad(const __grid_const
     }
     PhiStats st;
     {
-        const PhiStats mine = phi_stats_chunks(tl + kColU, uj0, uj1);
         float *o = x1 + (part * 128 + lr) * 8;
-        o[0] = mine.mp; o[1] = mine.sp; o[2] = mine.mn; o[3] = mine.sn;
-        if (kQuery) {
+        if (sub == 0) sign_stats_chunks<false>(tl + kColU, uj0, uj1, o);
+        else sign_stats_chunks<true>(tl + kColU, uj0, uj1, o + 2);
+        if (kQuery && sub == 1) {
             // scores: this part's 16-column chunks j = part, part + 2, ..: m, sum e^(s - m), sum e^(s - m) g.v
             float m = -INFINITY, l = 0.f, an = 0.f;
             for (int j = part; j < B / 16; j += 2) {
@@ -673,7 +705,7 @@ __global__ void __launch_bounds__(kGradThreads, 1) k_phi_grad(const __grid_const
             }
             o[4] = m; o[5] = l; o[6] = an;
         }
-        named_bar(pair_bar, 64);
+        named_bar(pair_bar, 128);
         const float *o0 = x1 + lr * 8, *o1 = x1 + (128 + lr) * 8;
         st = combine_stats(PhiStats{o0[0], o0[1], o0[2], o0[3]}, PhiStats{o1[0], o1[1], o1[2], o1[3]});
     }
@@ -683,25 +715,40 @@ __global__ void __launch_bounds__(kGradThreads, 1) k_phi_grad(const __grid_const
     // gives g.o = w A + Lambda and dw = lambda A - beta Lambda (= dN.sm_num + dD sm_den).
     float inv = 0.f, A = 0.f, beta = 0.f, lambda = 0.f;
     if (kQuery) {
-        // phi(q) of this part's columns into its operand image; partial lin_den = phi(q) . z
-        float ld = 0.f;
-        {
-            float x[32], yp[32], yn[32];
-            for (int j = uj0; j < uj1; ++j) {
-                tmem_ld32(tl + kColU + 32 * j, x);
+        // phi(q) of this thread's columns into its operand image; partial lin_den = phi(q) . z,
+        // one running sum over the part's columns, handed from sub 0 to sub 1
+        float zt[2][16];
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+            if (p < np) {
+                float x[16], yp[16], yn[16];
+                const int c0 = uc0 + 16 * p;
+                tmem_ld16(tl + kColU + c0, x);
                 tmem_wait_ld();
 #pragma unroll
-                for (int k = 0; k < 32; ++k) {
+                for (int k = 0; k < 16; ++k) {
                     yp[k] = valid ? ex2((x[k] - st.mp) * kLog2e) * ip : 0.f;
                     yn[k] = valid ? ex2((st.mn - x[k]) * kLog2e) * in : 0.f;
-                    ld += yp[k] * sZ[32 * j + k] + yn[k] * sZ[F + 32 * j + k];
+                    zt[p][k] = yp[k] * sZ[c0 + k] + yn[k] * sZ[F + c0 + k];
                 }
-                store_row32_bf16(smem + Lr.off_phi, 128 * 128, lr, 32 * j, yp);
-                store_row32_bf16(smem + Lr.off_phi, 128 * 128, lr, F + 32 * j, yn);
+                store_row_bf16(smem + Lr.off_phi, 128 * 128, lr, c0, yp);
+                store_row_bf16(smem + Lr.off_phi, 128 * 128, lr, F + c0, yn);
             }
         }
+        float ld = 0.f;
+        if (sub == 1) {
+            named_bar(pair_bar, 128);
+            ld = x2[part * 128 + lr];
+        }
+#pragma unroll
+        for (int p = 0; p < 2; ++p)
+            if (p < np) {
+#pragma unroll
+                for (int k = 0; k < 16; ++k) ld += zt[p][k];
+            }
         x2[part * 128 + lr] = ld;
-        named_bar(pair_bar, 64);
+        if (sub == 0) named_bar(pair_bar, 128);
+        named_bar(pair_bar, 128);
         const float lin_den = x2[lr] + x2[128 + lr];
         // scores of the whole row: shift c, D' = w sum_j e^(s_j - c) + lin_den e^(-c) (D = e^c D')
         const float *o0 = x1 + lr * 8, *o1 = x1 + (128 + lr) * 8;
@@ -717,55 +764,37 @@ __global__ void __launch_bounds__(kGradThreads, 1) k_phi_grad(const __grid_const
         beta = l * pw;
         lambda = lin_den * inv;
         A = an * pw;                              // sum_j (e^(s_j) / D) g.v_j
-        // dN = g / D of this part's half of the columns: Tensor Memory (fp32, A operand
-        // of S dN) and the operand image (bf16); its d/2 values are loaded at once
-        const uint4 *grow = reinterpret_cast<const uint4 *>(a.dO + (t0 + tok) * q_row + (size_t)(g * G + hl) * d) +
-                            part * (d / 16);
-        uint4 graw[8];
+        // dN = g / D of this thread's 32 columns: Tensor Memory (fp32, A operand of S dN) and
+        // the operand image (bf16)
+        if (sub < d / 64) {
+            float gv[32];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) graw[i] = (valid && i < d / 16) ? __ldg(grow + i) : make_uint4(0, 0, 0, 0);
+            for (int i = 0; i < 4; ++i) {
+                const uint32_t w4[4] = {graw[i].x, graw[i].y, graw[i].z, graw[i].w};
 #pragma unroll
-        for (int cc = 0; cc < 2; ++cc) {
-            if (cc < d / 64) {
-                float gv[32];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const uint4 q4 = graw[4 * cc + i];
-                    const uint32_t w4[4] = {q4.x, q4.y, q4.z, q4.w};
-#pragma unroll
-                    for (int jj = 0; jj < 4; ++jj) {
-                        gv[8 * i + 2 * jj] = __uint_as_float(w4[jj] << 16) * inv;
-                        gv[8 * i + 2 * jj + 1] = __uint_as_float(w4[jj] & 0xFFFF0000u) * inv;
-                    }
+                for (int jj = 0; jj < 4; ++jj) {
+                    gv[8 * i + 2 * jj] = __uint_as_float(w4[jj] << 16) * inv;
+                    gv[8 * i + 2 * jj + 1] = __uint_as_float(w4[jj] & 0xFFFF0000u) * inv;
                 }
-                const int col = part * (d / 2) + 32 * cc;
-                tmem_st32(tl + kColY + col, gv);
-                store_row32_bf16(smem + Lr.off_y, 128 * 128, lr, col, gv);
             }
+            tmem_st32(tl + kColY + ycol, gv);
+            store_row_bf16(smem + Lr.off_y, 128 * 128, lr, ycol, gv);
         }
     } else {
-        // V rows (fp32, this part's half of the columns) as the Tensor Memory A operand of
-        // R v; r enters with coefficient 1
-        const uint4 *vrow = reinterpret_cast<const uint4 *>(a.V + (t0 + tok) * kv_row + (size_t)g * d) + part * (d / 16);
-        uint4 vraw[8];
+        // V rows (fp32, this thread's 32 columns) as the Tensor Memory A operand of R v; r
+        // enters with coefficient 1
+        if (sub < d / 64) {
+            float vv[32];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) vraw[i] = (valid && i < d / 16) ? __ldg(vrow + i) : make_uint4(0, 0, 0, 0);
+            for (int i = 0; i < 4; ++i) {
+                const uint32_t w4[4] = {graw[i].x, graw[i].y, graw[i].z, graw[i].w};
 #pragma unroll
-        for (int cc = 0; cc < 2; ++cc) {
-            if (cc < d / 64) {
-                float vv[32];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const uint4 q4 = vraw[4 * cc + i];
-                    const uint32_t w4[4] = {q4.x, q4.y, q4.z, q4.w};
-#pragma unroll
-                    for (int jj = 0; jj < 4; ++jj) {
-                        vv[8 * i + 2 * jj] = __uint_as_float(w4[jj] << 16);
-                        vv[8 * i + 2 * jj + 1] = __uint_as_float(w4[jj] & 0xFFFF0000u);
-                    }
+                for (int jj = 0; jj < 4; ++jj) {
+                    vv[8 * i + 2 * jj] = __uint_as_float(w4[jj] << 16);
+                    vv[8 * i + 2 * jj + 1] = __uint_as_float(w4[jj] & 0xFFFF0000u);
                 }
-                tmem_st32(tl + kColY + part * (d / 2) + 32 * cc, vv);
             }
+            tmem_st32(tl + kColY + ycol, vv);
         }
     }
     tmem_wait_st();
@@ -777,24 +806,34 @@ __global__ void __launch_bounds__(kGradThreads, 1) k_phi_grad(const __grid_const
     // ---- dphi = [S | z] [dN; dD] (query) or [R | r] [v; 1] (key): tiles of 32 e ----
     if (!failed1 && tid == 0) {
         const uint32_t idC = instr_desc(FMT_TF32, FMT_TF32, false, false, 128, 2 * F);
-        for (int c = 0; c < NCHUNK && ok; ++c) {
-            const int slot = c & 1;
-            ok = wait_bar(&full[slot], (uint32_t)(c >> 1) & 1u, fail);
+        for (int q = 0; q < n_tiles && ok; ++q) {
+            const int slot = q % kGradSlots, b = q / NCHUNK, c = q - b * NCHUNK;
+            ok = wait_bar(&full[slot], (uint32_t)(q / kGradSlots) & 1u, fail);
             if (!ok) break;
             tc_fence_after();
             const uint32_t s_u = ring_u + slot * Lr.ring_slot;
+            // key side: block b's tiles write its own B lanes only
+            uint32_t off[4] = {0u, 0u, 0u, 0u};
+            if (!kQuery) {
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk)
-                mma_tf32_ts(tmem + kColG, tmem + kColY + 32 * c + 8 * kk, smem_desc(s_u + 32 * kk, 16, 1024, SWZ_128B),
-                            idC, (c | kk) != 0);
+                for (int w4 = 0; w4 < 4; ++w4) {
+                    const int lo = min(max(b * B - 32 * w4, 0), 32), hi = min(max((b + 1) * B - 32 * w4, 0), 32);
+                    off[w4] = hi <= lo ? 0xFFFFFFFFu : ~((0xFFFFFFFFu >> (32 - (hi - lo))) << lo);
+                }
+            }
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) {
+                const uint32_t ya = tmem + kColY + 32 * c + 8 * kk;
+                const uint64_t sb = smem_desc(s_u + 32 * kk, 16, 1024, SWZ_128B);
+                if (kQuery) mma_tf32_ts(tmem + kColG, ya, sb, idC, (c | kk) != 0);
+                else mma_tf32_ts_lanes(tmem + kColG, ya, sb, idC, off, (c | kk) != 0);
+            }
             mma_commit(&empty[slot]);
-            if (c + 2 < NCHUNK) {
-                ok = wait_bar(&empty[slot], (uint32_t)(c >> 1) & 1u, fail);
+            // the previous tile's slot, once its MMAs are done
+            if (q >= 1 && q - 1 + kGradSlots < n_tiles) {
+                ok = wait_bar(&empty[(q - 1) % kGradSlots], (uint32_t)((q - 1) / kGradSlots) & 1u, fail);
                 if (!ok) break;
-                mbar_arrive_expect_tx(&full[slot], Lr.ring_slot);
-                bulk_g2s(smem + ring_off + slot * Lr.ring_slot, src + (size_t)(c + 2) * 64 * F, Lr.ring_slot,
-                         &full[slot]);
-                ++loads_issued;
+                load_tile(q - 1 + kGradSlots);
             }
         }
         mma_commit(mbar);
@@ -810,28 +849,35 @@ __global__ void __launch_bounds__(kGradThreads, 1) k_phi_grad(const __grid_const
     // G = S dN (query) or R v (key) and zeta = z_{n-1} (query) or r_m (key); each part
     // takes its half of the features ----
     if (!failedC) {
-        float x[32], gp[32], gn[32];
-        // pass 0: Lambda+- = <G+-, p+->, Z+- = <zeta+-, p+-> over this part's features
-        float Lp = 0.f, Ln = 0.f, Zp = 0.f, Zn = 0.f;
+        // pass 0: Lambda+- = <G+-, p+->, Z+- = <zeta+-, p+-> over this part's features of one sign
+        float L = 0.f, Z = 0.f;
         for (int j = uj0; j < uj1; ++j) {
+            float x[32], gs[32];
             tmem_ld32(tl + kColU + 32 * j, x);
-            tmem_ld32(tl + kColG + 32 * j, gp);
-            tmem_ld32(tl + kColG + F + 32 * j, gn);
+            tmem_ld32(tl + kColG + sub * F + 32 * j, gs);
             tmem_wait_ld();
+            if (sub == 0) {
 #pragma unroll
-            for (int k = 0; k < 32; ++k) {
-                const float pp = ex2((x[k] - st.mp) * kLog2e) * ip;
-                const float pn = ex2((st.mn - x[k]) * kLog2e) * in;
-                Lp += gp[k] * pp;
-                Ln += gn[k] * pn;
-                Zp += sZ[32 * j + k] * pp;
-                Zn += sZ[F + 32 * j + k] * pn;
+                for (int k = 0; k < 32; ++k) {
+                    const float pp = ex2((x[k] - st.mp) * kLog2e) * ip;
+                    L += gs[k] * pp;
+                    Z += zr[32 * j + k] * pp;
+                }
+            } else {
+#pragma unroll
+                for (int k = 0; k < 32; ++k) {
+                    const float pn = ex2((st.mn - x[k]) * kLog2e) * in;
+                    L += gs[k] * pn;
+                    Z += zr[F + 32 * j + k] * pn;
+                }
             }
         }
+        float Lp, Ln, Zp, Zn;
         {
             float *o = x3 + (part * 128 + lr) * 4;
-            o[0] = Lp; o[1] = Ln; o[2] = Zp; o[3] = Zn;
-            named_bar(pair_bar, 64);
+            o[sub] = L;
+            o[2 + sub] = Z;
+            named_bar(pair_bar, 128);
             const float *o0 = x3 + lr * 4, *o1 = x3 + (128 + lr) * 4;
             Lp = o0[0] + o1[0];
             Ln = o0[1] + o1[1];
@@ -842,7 +888,7 @@ __global__ void __launch_bounds__(kGradThreads, 1) k_phi_grad(const __grid_const
         if (kQuery) {
             const float Lam = Lp + Ln;
             dD = -(w * A + Lam) * inv;   // -(g . o) / D
-            if (part == 0) {
+            if (part == 0 && sub == 0) {
                 sRowDw[lr] = valid ? lambda * A - beta * Lam : 0.f;
                 // column d of [dN | dD | 0] (the rest of that 32-column group is never read)
                 uint8_t *base = smem + Lr.off_y + (uint32_t)(d >> 6) * (128 * 128);
@@ -854,27 +900,29 @@ __global__ void __launch_bounds__(kGradThreads, 1) k_phi_grad(const __grid_const
             }
         }
         const float dotp = Lp + dD * Zp, dotn = Ln + dD * Zn;
-        // pass 1: du of this part's features
-        for (int j = uj0; j < uj1; ++j) {
-            tmem_ld32(tl + kColU + 32 * j, x);
-            tmem_ld32(tl + kColG + 32 * j, gp);
-            tmem_ld32(tl + kColG + F + 32 * j, gn);
+        // pass 1: du of this thread's columns
+#pragma unroll 1
+        for (int p = 0; p < np; ++p) {
+            float x[16], gp[16], gn[16], du[16];
+            const int c0 = uc0 + 16 * p;
+            tmem_ld16(tl + kColU + c0, x);
+            tmem_ld16(tl + kColG + c0, gp);
+            tmem_ld16(tl + kColG + F + c0, gn);
             tmem_wait_ld();
-            float du[32];
 #pragma unroll
-            for (int k = 0; k < 32; ++k) {
+            for (int k = 0; k < 16; ++k) {
                 const float pp = ex2((x[k] - st.mp) * kLog2e) * ip;
                 const float pn = ex2((st.mn - x[k]) * kLog2e) * in;
-                const float g1 = gp[k] + sZ[32 * j + k] * dD;
-                const float g2 = gn[k] + sZ[F + 32 * j + k] * dD;
+                const float g1 = gp[k] + zr[c0 + k] * dD;
+                const float g2 = gn[k] + zr[F + c0 + k] * dD;
                 du[k] = pp * (g1 - dotp) - pn * (g2 - dotn);
             }
             if (valid) {
                 bf16 *out = kQuery ? a.dUq + ((t0 + tok) * Hq + (size_t)(g * G + hl)) * F
                                    : a.dUk + ((t0 + tok) * Hkv + (size_t)g) * F;
-                uint4 *o4 = reinterpret_cast<uint4 *>(out + 32 * j);
+                uint4 *o4 = reinterpret_cast<uint4 *>(out + c0);
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
+                for (int q = 0; q < 2; ++q) {
                     uint4 v;
                     v.x = pack_bf16x2(du[8 * q + 0], du[8 * q + 1]);
                     v.y = pack_bf16x2(du[8 * q + 2], du[8 * q + 3]);
@@ -914,18 +962,16 @@ __global__ void __launch_bounds__(kGradThreads, 1) k_phi_grad(const __grid_const
         ok = wait_bar(mbar, 0, fail);
         tc_fence_after();
         // R's slot: per e-tile c the 2F feature rows (2F x 128 bytes, contiguous in global
-        // memory) are staged in the space of phi(Q) and [dN | dD], which the dR MMAs have
-        // consumed, laid out as in global memory, and written by bulk copies
+        // memory) are staged in the ring's slots and phi(Q)'s space, which the MMAs have
+        // consumed, laid out as in global memory, and written by bulk copies; the subs take
+        // alternate tiles
         if (!group_sync_failed(1, kGradThreads, !ok)) {
             float *R = a.R + (((size_t)s * a.n_blk + n) * Hkv + g) * hf;
             const uint32_t tile_bytes = (uint32_t)2 * F * 128;
-            for (int c = 0; c < d / 32; ++c) {
-                // buffers: phi's space (two tiles), then [dN | dD]'s; tile 3 reuses the first
-                uint8_t *buf = (c % 3 == 2) ? smem + Lr.off_y : smem + Lr.off_phi + (uint32_t)(c % 3) * tile_bytes;
-                if (c == 3) {
-                    if (tid == 0) bulk_wait_read_all();
-                    __syncthreads();
-                }
+            const bool issuer = part == 0 && lr == 0;
+#pragma unroll 1
+            for (int c = sub; c < d / 32; c += 2) {
+                uint8_t *buf = c < kGradSlots ? smem + Lr.off_ring + (uint32_t)c * Lr.ring_slot : smem + Lr.off_phi;
                 // part p stages the features of M-block p (with one block, part 0 alone)
                 for (int i = part; i < NM; i += 2) {
                     const int f = 128 * i + lr;
@@ -938,19 +984,20 @@ __global__ void __launch_bounds__(kGradThreads, 1) k_phi_grad(const __grid_const
                         row[q ^ (f & 7)] = make_float4(x[4 * q], x[4 * q + 1], x[4 * q + 2], x[4 * q + 3]);
                 }
                 fence_proxy_async_smem();
-                __syncthreads();
-                if (tid == 0) {
+                named_bar(6 + sub, kGradThreads / 2);
+                if (issuer) {
                     bulk_s2g(R + (size_t)c * 64 * F, buf, tile_bytes);
                     bulk_commit();
                 }
             }
-            for (int i = part; i < NM; i += 2) {
-                float zz[16];
-                tmem_ld16(tl + kColDR + (uint32_t)(i * NYS + d), zz);
-                tmem_wait_ld();
-                R[z_offset(128 * i + lr, d, F)] = zz[0];
-            }
-            if (tid == 0) bulk_wait_all();
+            if (sub == 1)
+                for (int i = part; i < NM; i += 2) {
+                    float zz[16];
+                    tmem_ld16(tl + kColDR + (uint32_t)(i * NYS + d), zz);
+                    tmem_wait_ld();
+                    R[z_offset(128 * i + lr, d, F)] = zz[0];
+                }
+            if (issuer) bulk_wait_all();
         } else {
             ok = false;
         }
@@ -958,10 +1005,8 @@ __global__ void __launch_bounds__(kGradThreads, 1) k_phi_grad(const __grid_const
     if (tid == 0 && (failed2 || !ok)) raise_error(a.err, ERR_WAIT_TIMEOUT);
     // no tile copy may still be landing when the CTA leaves
     if (tid == 0) {
-        for (int c = 0; c < loads_issued; ++c) {
-            // loads c and c+2 share slot c&1; the later one completes the later phase
-            if (c + 2 >= loads_issued) mbar_wait(&full[c & 1], (uint32_t)(c >> 1) & 1u, kWaitNs);
-        }
+        for (int q = max(0, loads_issued - kGradSlots); q < loads_issued; ++q)
+            mbar_wait(&full[q % kGradSlots], (uint32_t)(q / kGradSlots) & 1u, kWaitNs);
     }
     tc_fence_before();
     __syncthreads();
@@ -1318,6 +1363,7 @@ cudaError_t launch_train_backward(const hybrid_cfg &c, const void *Q, const void
             return cudaErrorInvalidValue;
     }
     const int units = n_seq * a.n_blk * a.Hkv;
+    const int nbk = 128 / a.B, key_units = n_seq * ((a.n_blk + nbk - 1) / nbk) * a.Hkv;   // 128 keys per CTA
     const size_t sf = slot_floats(a.Hkv, a.d, a.F);
     cudaError_t e;
     const RowLayout Lg = make_grad_layout(a.d, a.F, a.B);
@@ -1330,7 +1376,7 @@ cudaError_t launch_train_backward(const hybrid_cfg &c, const void *Q, const void
     if ((e = launch_pdl(k_slot_scan, dim3((unsigned)((n4 + 255) / 256), 1), dim3(256), 0, st, a.R,
                         static_cast<float *>(nullptr), n_seq, a.n_blk, sf, true)) != cudaSuccess)
         return e;
-    if ((e = launch_pdl(k_phi_grad<false>, dim3((unsigned)units), dim3(kGradThreads), Lg.bytes, st, a, Lg)) !=
+    if ((e = launch_pdl(k_phi_grad<false>, dim3((unsigned)key_units), dim3(kGradThreads), Lg.bytes, st, a, Lg)) !=
         cudaSuccess)
         return e;
     DwArgs b{};
