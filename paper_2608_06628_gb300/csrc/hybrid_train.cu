@@ -70,6 +70,7 @@ struct TrainArgs {
     float *dap;   // per (sequence, block, state head): the G gate terms, summed by k_grad_reduce
     unsigned *err;
     int n_seq, L, B, Hq, Hkv, d, F, n_blk;
+    int nbk;   // blocks per CTA of the key side
 };
 
 // Partial sums of dW kept for the ordered reduction: at most this many CTAs of
@@ -113,39 +114,14 @@ __device__ __forceinline__ void store_row_bf16(uint8_t *img, uint32_t pstride, i
     }
 }
 
-// Row statistics of phi = [softmax(u), softmax(-u)] for the F values of u in
-// Tensor Memory columns [col, col + F) of this thread's lane.
+// Row statistics of phi = [softmax(u), softmax(-u)] for the F values of u in Tensor Memory.
 struct PhiStats {
     float mp, sp, mn, sn;   // max u, sum e^(u - mp), min u, sum e^(mn - u)
 };
-__device__ __forceinline__ PhiStats phi_stats(uint32_t taddr, int F)
-{
-    PhiStats s{-INFINITY, 0.f, INFINITY, 0.f};
-    float x[32];
-    for (int j = 0; j < F / 32; ++j) {
-        ptx::tmem_ld32(taddr + 32 * j, x);
-        ptx::tmem_wait_ld();
-#pragma unroll
-        for (int k = 0; k < 32; ++k) {
-            s.mp = fmaxf(s.mp, x[k]);
-            s.mn = fminf(s.mn, x[k]);
-        }
-    }
-    for (int j = 0; j < F / 32; ++j) {
-        ptx::tmem_ld32(taddr + 32 * j, x);
-        ptx::tmem_wait_ld();
-#pragma unroll
-        for (int k = 0; k < 32; ++k) {
-            s.sp += ex2((x[k] - s.mp) * kLog2e);
-            s.sn += ex2((s.mn - x[k]) * kLog2e);
-        }
-    }
-    return s;
-}
 
-// Partial statistics of one sign over the 32-column chunks [j0, j1) only, to be
-// combined with the other chunks' by combine_stats: max u and sum e^(u - max), or
-// min u and sum e^(min - u).
+// Statistics of one sign over the 32-column chunks [j0, j1) of u at taddr (partial ones are
+// combined with the other chunks' by combine_stats): max u and sum e^(u - max), or min u and
+// sum e^(min - u).
 template <bool kNeg>
 __device__ __forceinline__ void sign_stats_chunks(uint32_t taddr, int j0, int j1, float *out)
 {
@@ -233,6 +209,10 @@ __device__ __forceinline__ uint8_t *aligned_smem(uint8_t *raw)
 // increments of the group's blocks into their own Tensor Memory columns (one
 // commit), then per block: store the running state (registers, thread = e)
 // into its slot and add the block's increment.
+// What bounds it: the two images' stores (32 KB a block and slice, bulk copies), while the
+// other phases of a group wait for each other; the softmax sums of the slice's sign only and
+// the next group's rows brought into L2 took 88 us to 84 (8 sequences x 1024 tokens, four
+// state heads, d = F = 128: 270 MB).
 // Shared memory: W, K rows, V rows (two panels of 64 e, the second zero for
 // d = 64, so that V^T is an M = 128 operand), phi slice, row scratch (in K's
 // space); 107 KB and 256 Tensor Memory columns, so two CTAs share an SM.
@@ -329,6 +309,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_prefix_states(const __grid_cons
             if (b0 == 0)
                 for (int p = 0; p < F / 64; ++p)
                     tma_load_2d(smem + Lp.off_w + p * d * 128, &a.tmW, 64 * p, g * d, tbar);
+            // the next group's rows into L2 meanwhile
+            if (b0 + GB < n_blk)
+                for (int p = 0; p < d / 64; ++p) {
+                    tma_prefetch_3d(&a.tmKg, 64 * p, g, (int)t0 + GB * B);
+                    tma_prefetch_3d(&a.tmVg, 64 * p, g, (int)t0 + GB * B);
+                }
         }
         ok = wait_bar(tbar, (uint32_t)(b0 / GB) & 1u, fail) && ok;
         tc_fence_before();
@@ -347,15 +333,17 @@ __global__ void __launch_bounds__(kThreads, 1) k_prefix_states(const __grid_cons
         // the slice of phi of row tid (full-F softmax statistics), bf16 into the
         // [feature][token] operand and fp32 into the row scratch
         {
-            const PhiStats st = phi_stats(tmem + lane_off, F);
-            const float inv = 1.f / (neg ? st.sn : st.sp);
+            float st[2];   // the slice's sign only
+            if (neg) sign_stats_chunks<true>(tmem + lane_off, 0, F / 32, st);
+            else sign_stats_chunks<false>(tmem + lane_off, 0, F / 32, st);
+            const float inv = 1.f / st[1];
             float x[32];
             tmem_ld32(tmem + lane_off + (uint32_t)fu, x);
             tmem_wait_ld();
             const bool valid = tid < nt;
 #pragma unroll
             for (int k = 0; k < 32; ++k) {
-                const float ph = valid ? ex2((neg ? (st.mn - x[k]) : (x[k] - st.mp)) * kLog2e) * inv : 0.f;
+                const float ph = valid ? ex2((neg ? (st[0] - x[k]) : (x[k] - st[0])) * kLog2e) * inv : 0.f;
                 xs[tid * 32 + ((k + tid) & 31)] = ph;   // rotated: conflict-free across the warp
                 const __nv_bfloat16 hb = __float2bfloat16_rn(ph);
                 uint8_t *row = smem + Lp.off_p + (uint32_t)(tid >> 6) * (32 * 128) + (uint32_t)k * 128u;
@@ -500,9 +488,9 @@ __global__ void k_slot_scan(float *buf0, float *buf1, int n_seq, int n_slots, si
 }
 
 // ---------------------------------------------------------------------------
-// k_phi_grad<kQuery>: sequence s, state head g, block n (query side) or the 128 / B blocks
-// from n on (key side).  On the key side a block fills B of the 128 rows, so a CTA takes as
-// many blocks as fit: the row arithmetic is done once for all of them, each block's R tiles
+// k_phi_grad<kQuery>: sequence s, state head g, block n (query side) or up to 128 / B blocks
+// from n on (key side).  On the key side a block fills B of the 128 rows, so a CTA takes
+// several blocks (launch_train_backward chooses how many): the row arithmetic is done once for all of them, each block's R tiles
 // multiply all rows, and the lanes of the other blocks are left out of that product's result.
 // What bounds it: the phases of a CTA follow one another (one CTA per SM: the operands and
 // tiles take its shared memory, a row's products its Tensor Memory), the key side also the
@@ -523,8 +511,8 @@ __global__ void __launch_bounds__(kGradThreads, 1) k_phi_grad(const __grid_const
     // half of the part's columns; warps w, w + 4, .. share lanes 32 (w & 3) ..
     const int lr = tid & 127, part = (tid >> 7) & 1, sub = tid >> 8;
     const int d = a.d, F = a.F, B = a.B, Hkv = a.Hkv, Hq = a.Hq, G = Hq / Hkv;
-    // blocks [n, n + nb) of sequence s: one on the query side, up to 128 rows on the key side
-    const int nbk = kQuery ? 1 : 128 / B, n_grp = (a.n_blk + nbk - 1) / nbk;
+    // blocks [n, n + nb) of sequence s: one on the query side, a group of up to nbk on the key side
+    const int nbk = kQuery ? 1 : a.nbk, n_grp = (a.n_blk + nbk - 1) / nbk;
     const int g = blockIdx.x % Hkv, n = (blockIdx.x / Hkv) % n_grp * nbk, s = blockIdx.x / (Hkv * n_grp);
     const int nb = min(nbk, a.n_blk - n);
     // Rows of the tile on Tensor Memory lanes: query side, lane r < G*B is token r / G,
@@ -1149,31 +1137,53 @@ __global__ void __launch_bounds__(kThreads, 1) k_dw(const __grid_constant__ DwAr
 // ---------------------------------------------------------------------------
 // k_grad_reduce: dW[g] = sum over parts p = 0, 1, ... of dWp[g][p] and
 // d alpha[g G + h] = sum over blocks u = 0, 1, ... of dap[u][g][h], each in that order.
+// What bounds it: the latency of the loads.  A warp of d alpha has 256 blocks in flight,
+// eight per lane, which lane 0 then adds one after the other: with one thread's loads behind
+// its adds, forward and backward of 8 sequences x 1024 tokens, 16:4 heads, took 419 us
+// (32 loads in flight in that thread: 415), with this 408.
 // ---------------------------------------------------------------------------
 struct ReduceArgs {
     const float *dWp, *dap;
     float *dW, *dalpha;
-    int Hkv, G, dF, parts, blocks;   // dF = d * F; blocks = n_seq * n_blk
+    int Hkv, G, dF, parts, blocks, w_ctas;   // dF = d * F; blocks = n_seq * n_blk
 };
 
-__global__ void k_grad_reduce(const ReduceArgs a)
+// CTAs [0, w_ctas): dW, an element per thread; the others: d alpha, an element per warp
+__global__ void __launch_bounds__(256) k_grad_reduce(const ReduceArgs a)
 {
     using namespace ptx;
+    __shared__ float sV[8][256];
     griddep_wait();
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long nw = (long long)a.Hkv * a.dF;
-    if (i < nw) {
-        const int g = (int)(i / a.dF);
-        const long long e = i % a.dF;
-        const float *p = a.dWp + (long long)g * a.parts * a.dF + e;
-        float sum = 0.f;
-        for (int k = 0; k < a.parts; ++k) sum += p[(long long)k * a.dF];
-        a.dW[i] = sum;
-    } else if (i < nw + (long long)a.Hkv * a.G) {
-        const int j = (int)(i - nw);   // g G + h
-        float sum = 0.f;
-        for (int u = 0; u < a.blocks; ++u) sum += a.dap[(long long)u * a.Hkv * a.G + j];
-        a.dalpha[j] = sum;
+    if ((int)blockIdx.x < a.w_ctas) {
+        const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+        if (i < (long long)a.Hkv * a.dF) {
+            const int g = (int)(i / a.dF);
+            const float *p = a.dWp + (long long)g * a.parts * a.dF + i % a.dF;
+            float sum = 0.f;
+            for (int k = 0; k < a.parts; ++k) sum += p[(long long)k * a.dF];
+            a.dW[i] = sum;
+        }
+    } else {
+        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, Hq = a.Hkv * a.G;
+        const int j = ((int)blockIdx.x - a.w_ctas) * 8 + warp;   // g G + h
+        if (j < Hq) {
+            float sum = 0.f;
+            for (int u0 = 0; u0 < a.blocks; u0 += 256) {
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    const int u = u0 + 32 * k + lane;
+                    sV[warp][32 * k + lane] = u < a.blocks ? a.dap[(long long)u * Hq + j] : 0.f;
+                }
+                __syncwarp();
+                if (lane == 0) {
+                    const int nu = min(256, a.blocks - u0);
+#pragma unroll 16
+                    for (int k = 0; k < nu; ++k) sum += sV[warp][k];
+                }
+                __syncwarp();
+            }
+            if (lane == 0) a.dalpha[j] = sum;
+        }
     }
     griddep_launch_dependents();
 }
@@ -1363,7 +1373,15 @@ cudaError_t launch_train_backward(const hybrid_cfg &c, const void *Q, const void
             return cudaErrorInvalidValue;
     }
     const int units = n_seq * a.n_blk * a.Hkv;
-    const int nbk = 128 / a.B, key_units = n_seq * ((a.n_blk + nbk - 1) / nbk) * a.Hkv;   // 128 keys per CTA
+    // Key side: the group size with the least waves x (3 + blocks): a CTA's fixed phases take
+    // as long as three blocks' tiles (12.3 us with one block of 32, 22 with four, d = F = 128),
+    // and a short batch spreads its blocks over the SMs.
+    auto groups = [&](int nbk) { return (long long)n_seq * ((a.n_blk + nbk - 1) / nbk) * a.Hkv; };
+    auto cost = [&](int nbk) { return (groups(nbk) + sm_count() - 1) / sm_count() * (3 + nbk); };
+    a.nbk = 1;
+    for (int k = 2; k <= 128 / a.B; ++k)
+        if (cost(k) < cost(a.nbk)) a.nbk = k;
+    const long long key_units = groups(a.nbk);
     const size_t sf = slot_floats(a.Hkv, a.d, a.F);
     cudaError_t e;
     const RowLayout Lg = make_grad_layout(a.d, a.F, a.B);
@@ -1416,8 +1434,8 @@ cudaError_t launch_train_backward(const hybrid_cfg &c, const void *Q, const void
     rd.dF = a.d * a.F;
     rd.parts = per_group;
     rd.blocks = a.n_seq * a.n_blk;
-    const long long n_out = (long long)a.Hkv * rd.dF + a.Hq;
-    return launch_pdl(k_grad_reduce, dim3((unsigned)((n_out + 255) / 256)), dim3(256), 0, st, rd);
+    rd.w_ctas = (int)(((long long)a.Hkv * rd.dF + 255) / 256);
+    return launch_pdl(k_grad_reduce, dim3((unsigned)(rd.w_ctas + (a.Hq + 7) / 8)), dim3(256), 0, st, rd);
 }
 
 }  // namespace hyb

@@ -10,11 +10,13 @@ from test_gpu_train import TOL, TW, inputs, run_gpu
 
 pytestmark = pytest.mark.gpu
 
+# the group size follows the number of blocks: 1 while they fit the SMs, then the least waves
 CASES = [
-    TW("b16_17_blocks", 2, 272, 4, 2, 64, 128, 16, 81),    # 8 + 8 + 1 blocks of 16
-    TW("b32_9_blocks", 2, 288, 8, 2, 128, 128, 32, 82),    # 4 + 4 + 1
-    TW("b64_5_blocks", 2, 320, 2, 1, 128, 64, 64, 83),     # 2 + 2 + 1
-    TW("b32_7_blocks", 3, 224, 2, 2, 64, 64, 32, 84),      # 4 + 3
+    TW("b16_groups_of_6", 40, 272, 4, 2, 64, 128, 16, 81),     # 17 blocks of 16: 6 + 6 + 5
+    TW("b16_groups_of_8", 50, 384, 2, 1, 64, 64, 16, 85),      # 24 blocks: 8 + 8 + 8
+    TW("b32_groups_of_4", 19, 416, 4, 2, 128, 128, 32, 82),    # 13 blocks of 32: 4 + 4 + 4 + 1
+    TW("b64_groups_of_2", 36, 320, 2, 1, 128, 64, 64, 83),     # 5 blocks of 64: 2 + 2 + 1
+    TW("b32_ungrouped", 3, 224, 2, 2, 64, 64, 32, 84),         # 42 blocks in all
 ]
 
 
