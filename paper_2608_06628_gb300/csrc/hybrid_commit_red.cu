@@ -195,14 +195,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_commit_red(const __grid_constan
         bool ok = true;
         for (int u = u_begin; u < u_end && ok; ++u) {
             const int Tu = unit_len(a, u);   // a request without tokens has no work
-            if (Tu == 0) continue;
+            if (Tu == 0 || !unit_head(a, u)) continue;
             const int n_chunks = (Tu + kChunk - 1) / kChunk;
             const long long tok0 = unit_tok0(a, u);
             const int g = (u / a.n_pass) % a.Hkv;
-            // the first chunk's keys on their way beside the state pointer
-            KtRegs kr;
-            kt_load(a.K, (size_t)tok0, min(kChunk, Tu), a.Hkv, g, d, kr, lane);
-            if (!unit_head(a, u)) continue;
             if (kp > 0) ok = wait_bar(wfree, (kp - 1) & 1u, fail);
             if (__any_sync(0xffffffffu, !ok)) break;
             if (lane == 0) {
@@ -213,8 +209,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_commit_red(const __grid_constan
             for (int j = 0; j < n_chunks; ++j, ++cc) {
                 const int b = cc & 1;
                 uint8_t *cb = smem + a.off_c + b * a.chunk_stride;
-                if (j > 0)
-                    kt_load(a.K, (size_t)tok0 + (size_t)j * kChunk, min(kChunk, Tu - j * kChunk), a.Hkv, g, d, kr, lane);
+                KtRegs kr;
+                kt_load(a.K, (size_t)tok0 + (size_t)j * kChunk, min(kChunk, Tu - j * kChunk), a.Hkv, g, d, kr, lane);
                 ok = wait_bar(&cfree[b], ((cc >> 1) & 1u) ^ 1u, fail);
                 if (__any_sync(0xffffffffu, !ok)) break;
                 if (lane == 0) {
@@ -301,7 +297,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_commit_red(const __grid_constan
     } else if (warp == 2) {
         // --------------------------------------------------------------- storer
         if (lane == 0) {
-            uint32_t kp = 0, sg = 0, rel = 0;   // units, tiles issued, tiles whose slot is released
+            uint32_t kp = 0, sg = 0;
             bool ok = true;
             for (int u = u_begin; u < u_end && ok; ++u) {
                 if (unit_len(a, u) == 0) continue;
@@ -313,16 +309,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_commit_red(const __grid_constan
                 bulk_commit();
                 bulk_wait_read_all();
                 mbar_arrive(dzfree);
-                for (; rel < sg; ++rel) mbar_arrive(&sempty[rel % kStage]);
-                // up to two tiles' reductions are on their way out while the next is staged
-                for (int c = 0; c < NCP; ++c) {
+                for (int c = 0; c < NCP; ++c, ++sg) {
                     const int slot = sg % kStage;
                     if (!wait_bar(&sfull[slot], (sg / kStage) & 1u, fail)) { ok = false; break; }
                     bulk_reduce_add_f32(Sg + (size_t)(pass * NCP + c) * 32 * d, stage + (size_t)slot * atom, atom);
                     bulk_commit();
-                    ++sg;
-                    bulk_wait_read_2();
-                    for (; rel + 2 < sg; ++rel) mbar_arrive(&sempty[rel % kStage]);
+                    bulk_wait_read_all();
+                    mbar_arrive(&sempty[slot]);
                 }
                 ++kp;
             }
