@@ -211,10 +211,6 @@ hybrid_status hybrid_block_attn_commit_logical(const hybrid_cfg *cfg, const void
     return from_cuda(hyb::launch_scratch_unpack(*cfg, states, n_req, S_logical, z_logical, stream));
 }
 
-// Commits of more tokens than this run the prefill kernel (measured crossover
-// on the batch-64 shape: 64 tokens per request).
-constexpr int kPrefillMinTokens = 64;
-
 hybrid_status hybrid_commit_block(const hybrid_cfg *cfg, const void *K, const void *V, int n_tok,
                                   const void *W, void *const *d_state_ptrs, int n_req,
                                   cudaStream_t stream)
@@ -228,9 +224,7 @@ hybrid_status hybrid_commit_block(const hybrid_cfg *cfg, const void *K, const vo
         return HYBRID_ERR_INVALID_ARG;
     unsigned *err = error_word();
     if (!err) return HYBRID_ERR_CUDA;
-    // block commits (a few dozen tokens) run the per-unit reduction kernel; longer
-    // prompts the token-major prefill kernel, which balances chunks across SMs
-    if (n_tok > kPrefillMinTokens && hyb::prefill_supported(*cfg))
+    if (hyb::commit_by_prefill(*cfg, n_tok, (long long)n_req * cfg->n_kv_heads))
         return from_cuda(hyb::launch_prefill(*cfg, K, V, n_tok, W, d_state_ptrs, n_req, err, stream));
     if (hyb::commit_red_supported(*cfg))
         return from_cuda(hyb::launch_commit_red(*cfg, K, V, n_tok, W, d_state_ptrs, n_req, err, stream));
@@ -278,10 +272,8 @@ hybrid_status hybrid_commit_ragged(const hybrid_cfg *cfg, const void *K, const v
         for (int i = 0; i < nb; ++i) longest = tok[i + 1] - tok[i] > longest ? tok[i + 1] - tok[i] : longest;
         if (tok[nb] == 0) continue;
         const size_t off = (size_t)tok_offsets[r0] * row_bytes;
-        // as for uniform prompts: the token-major kernel once a prompt is longer than a
-        // block commit (it balances chunks across SMs), else the per-unit reduction kernel
         const cudaError_t e =
-            pre && (longest > kPrefillMinTokens || !red)
+            hyb::commit_by_prefill(*cfg, longest, (long long)nb * cfg->n_kv_heads)
                 ? hyb::launch_prefill_ragged(*cfg, Kb + off, Vb + off, tok, W, d_state_ptrs + r0, nb, err, stream)
                 : hyb::launch_commit_red_ragged(*cfg, Kb + off, Vb + off, tok, W, d_state_ptrs + r0, nb, err, stream);
         if (e != cudaSuccess) return from_cuda(e);

@@ -193,7 +193,10 @@ struct ChunkWalk {
     }
 };
 
-template <class A>
+// kShort: commits of at most a block's 64 tokens form phi as k_commit_red does (the normaliser
+// added in halves of 32 features, phi = e^(..) / l), which committed them before and still does
+// where it is faster: the bf16 phi(K), and so the state, is the same from either kernel.
+template <class A, bool kShort>
 __global__ void __launch_bounds__(kThreads, 1) k_prefill(const __grid_constant__ A a)
 {
     using namespace ptx;
@@ -246,6 +249,16 @@ __global__ void __launch_bounds__(kThreads, 1) k_prefill(const __grid_constant__
     __syncthreads();
     tc_fence_after();
     if (tid == 0) griddep_launch_dependents();
+    // the K and V boxes of the CTA's first chunks into L2 while the previous kernel drains: a
+    // prefetch brings no value into the SM, so it needs no ordering after that kernel
+    if (tid == 64) {
+        int n = 0;
+        for (ChunkWalk<A> w(a, lo, hi); w.more() && n < 2; w.next(a), ++n) {
+            const ChunkPos p = w.pos(a);
+            tma_prefetch_4d(&a.tmK, 0, p.u % a.Hkv, p.row0, 0);
+            tma_prefetch_4d(&a.tmV, 0, p.u % a.Hkv, p.row0, 0);
+        }
+    }
     griddep_wait();
     const uint32_t tmem = *tmem_holder;
     uint8_t *stage = smem + a.off_s;
@@ -460,21 +473,37 @@ __global__ void __launch_bounds__(kThreads, 1) k_prefill(const __grid_constant__
                     tmem_ld32(ub + 32 * jj, reinterpret_cast<float(&)[32]>(x[0]));
                     tmem_ld32(ub + 32 * jj + 32, reinterpret_cast<float(&)[32]>(x[32]));
                     tmem_wait_ld();
+                    if constexpr (kShort) {
 #pragma unroll
-                    for (int t = 0; t < 64; ++t) l += ex2(fmaf(x[t], sgn, -m));
+                        for (int t = 0; t < 64; ++t) x[t] = ex2(fmaf(x[t], sgn, -m));
+#pragma unroll
+                        for (int w2 = 16; w2 >= 1; w2 >>= 1)
+#pragma unroll
+                            for (int t = 0; t < w2; ++t) {
+                                x[t] += x[t + w2];
+                                x[32 + t] += x[32 + t + w2];
+                            }
+                        l += x[0] + x[32];
+                    } else {
+#pragma unroll
+                        for (int t = 0; t < 64; ++t) l += ex2(fmaf(x[t], sgn, -m));
+                    }
                 }
             }
             // phi = 2^(sgn u - m) / l = 2^(sgn u - (m + log2 l)): the normaliser folds
             // into the exponent's offset
-            const float mo = m + __log2f(l);
+            const float mo = kShort ? m : m + __log2f(l), inv_l = kShort ? 1.f / l : 1.f;
             const bool full = 32 * q4 + 32 <= nt;   // warp-uniform: every token of the warp is valid
             // phi(K) is rewritten once the previous chunk's dS^T has read it
             if (i > 0) bad = !wait_bar(dsdone, (i - 1) & 1u, fail) || bad;
             if (active) {
                 // offsets of this thread's four tokens (8 i + lane / 4)
-                float mt4[4];
+                float mt4[4], il4[4];
 #pragma unroll
-                for (int i4 = 0; i4 < 4; ++i4) mt4[i4] = __shfl_sync(0xffffffffu, mo, 8 * i4 + (lane >> 2));
+                for (int i4 = 0; i4 < 4; ++i4) {
+                    mt4[i4] = __shfl_sync(0xffffffffu, mo, 8 * i4 + (lane >> 2));
+                    il4[i4] = kShort ? __shfl_sync(0xffffffffu, inv_l, 8 * i4 + (lane >> 2)) : 1.f;
+                }
 #pragma unroll 2
                 for (int jj = 0; jj < NCH; ++jj) {
                     // x[8 i + 2 j + h]: token 8 i + lane / 4, feature 8 j + 2 (lane mod 4) + h
@@ -485,7 +514,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_prefill(const __grid_constant__
 #pragma unroll
                     for (int i4 = 0; i4 < 4; ++i4)
 #pragma unroll
-                        for (int c = 0; c < 8; ++c) x[8 * i4 + c] = ex2(fmaf(x[8 * i4 + c], sgn, -mt4[i4]));
+                        for (int c = 0; c < 8; ++c) {
+                            const float ek = ex2(fmaf(x[8 * i4 + c], sgn, -mt4[i4]));
+                            x[8 * i4 + c] = kShort ? ek * il4[i4] : ek;
+                        }
                     if (!full) {
 #pragma unroll
                         for (int i4 = 0; i4 < 4; ++i4)
@@ -572,6 +604,22 @@ bool prefill_supported(const hybrid_cfg &c)
     return (int)make_playout(c.head_dim, c.feat_dim).bytes <= kSmemLimit;
 }
 
+// Which of the two tensor-core kernels folds prompts or blocks of up to `longest` tokens into
+// `units` states.  The token-major kernel, which balances chunks across SMs, is the faster one
+// (alone, us, 4 heads, against k_commit_red: d = F = 64, 40 requests of 32 tokens 8.9 against
+// 11.4, 256 requests 23.5 against 35.5; d = F = 128, 64 tokens, 57 requests 18.5 against 21.9;
+// after four steps of 64 requests, d = F = 128, 72.8 against 74.5 for the whole), except for up
+// to 32 tokens with d = F = 128 where whole waves of units fill most SMs: 112 units 11.8 against
+// 11.2, 152: 13.3 against 12.8, 304: 20.3 against 19.8, 456: 27.6 against 27.3 (but 76: 10.0
+// against 10.8, 1024: 55.6 against 57.4; 8 steps and the commit of 512: 194.8 against 201).
+bool commit_by_prefill(const hybrid_cfg &c, int longest, long long units)
+{
+    if (!prefill_supported(c)) return false;
+    if (!commit_red_supported(c) || longest > 32 || c.head_dim < 128 || c.feat_dim < 128) return true;
+    const int sms = sm_count();
+    return 2 * units <= sms || units > 3ll * sms;
+}
+
 namespace {
 
 // Tensor maps and sizes shared by the uniform and the ragged launch; rows = tokens of K and V.
@@ -606,7 +654,7 @@ bool fill_prefill_args(const hybrid_cfg &c, const void *K, const void *V, long l
     return true;
 }
 
-template <class A>
+template <class A, bool kShort>
 cudaError_t run_prefill(const hybrid_cfg &c, const A &a, long long total, cudaStream_t st)
 {
     if (total <= 0) return cudaSuccess;
@@ -618,7 +666,7 @@ cudaError_t run_prefill(const hybrid_cfg &c, const A &a, long long total, cudaSt
     const unsigned long long bit = 1ull << dev;
     if (!(opted.load(std::memory_order_acquire) & bit)) {
         const cudaError_t e =
-            cudaFuncSetAttribute(k_prefill<A>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
+            cudaFuncSetAttribute(k_prefill<A, kShort>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
         if (e != cudaSuccess) return e;
         opted.fetch_or(bit, std::memory_order_acq_rel);
     }
@@ -632,7 +680,7 @@ cudaError_t run_prefill(const hybrid_cfg &c, const A &a, long long total, cudaSt
     at[0].val.programmaticStreamSerializationAllowed = 1;
     lc.attrs = at;
     lc.numAttrs = 1;
-    return cudaLaunchKernelEx(&lc, k_prefill<A>, a);
+    return cudaLaunchKernelEx(&lc, k_prefill<A, kShort>, a);
 }
 
 }  // namespace
@@ -644,7 +692,9 @@ cudaError_t launch_prefill(const hybrid_cfg &c, const void *K, const void *V, in
     if (!fill_prefill_args(c, K, V, (long long)n_req * n_tok, W, states, n_req, err, a)) return cudaErrorInvalidValue;
     a.T = n_tok;
     a.n_chunks = (n_tok + kCT - 1) / kCT;
-    return run_prefill(c, a, (long long)a.n_units * a.n_chunks, st);
+    const long long total = (long long)a.n_units * a.n_chunks;
+    return n_tok <= kShortCommit ? run_prefill<PrefillArgs, true>(c, a, total, st)
+                                 : run_prefill<PrefillArgs, false>(c, a, total, st);
 }
 
 cudaError_t launch_prefill_ragged(const hybrid_cfg &c, const void *K, const void *V, const int *tok, const void *W,
@@ -660,7 +710,11 @@ cudaError_t launch_prefill_ragged(const hybrid_cfg &c, const void *K, const void
     a.ch[0] = 0;
     for (int r = 0; r <= n_req; ++r) a.tok[r] = tok[r];
     for (int r = 0; r < n_req; ++r) a.ch[r + 1] = a.ch[r] + (tok[r + 1] - tok[r] + kCT - 1) / kCT;
-    return run_prefill(c, a, (long long)c.n_kv_heads * a.ch[n_req], st);
+    int longest = 0;
+    for (int r = 0; r < n_req; ++r) longest = tok[r + 1] - tok[r] > longest ? tok[r + 1] - tok[r] : longest;
+    const long long total = (long long)c.n_kv_heads * a.ch[n_req];
+    return longest <= kShortCommit ? run_prefill<PrefillRaggedArgs, true>(c, a, total, st)
+                                   : run_prefill<PrefillRaggedArgs, false>(c, a, total, st);
 }
 
 }  // namespace hyb

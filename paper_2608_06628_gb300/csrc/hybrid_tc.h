@@ -55,6 +55,7 @@ bool commit_red_supported(const hybrid_cfg &c);
 // (hybrid_prefill.cu): 128-token chunks, ranges of chunks balanced across SMs,
 // increments added by bulk reduce-adds; any n_tok >= 1.
 bool prefill_supported(const hybrid_cfg &c);
+bool commit_by_prefill(const hybrid_cfg &c, int longest, long long units);   // rather than k_commit_red
 cudaError_t launch_prefill(const hybrid_cfg &c, const void *K, const void *V, int n_tok, const void *W,
                            void *const *states, int n_req, unsigned *err, cudaStream_t st);
 cudaError_t launch_commit_red(const hybrid_cfg &c, const void *K, const void *V, int n_tok, const void *W,
@@ -69,6 +70,9 @@ cudaError_t launch_phi_tc(const void *X, int n_rows, int nh, int Hkv, int d, int
 // [tok[n_req]][Hkv][d]; tok is a host array read at launch (its values travel in
 // the kernel parameters), so at most kMaxRaggedRequests requests per launch.
 constexpr int kMaxRaggedRequests = 2048;
+// Commits of at most this many tokens per request form phi(K) alike in the block-commit and the
+// prefill kernel (same bits).
+constexpr int kShortCommit = 64;
 cudaError_t launch_prefill_ragged(const hybrid_cfg &c, const void *K, const void *V, const int *tok, const void *W,
                                   void *const *states, int n_req, unsigned *err, cudaStream_t st);
 cudaError_t launch_commit_red_ragged(const hybrid_cfg &c, const void *K, const void *V, const int *tok,
