@@ -223,8 +223,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_prefill(const __grid_constant__
     uint64_t *dsdone = pready + 1;     // the chunk's dS^T products are complete (phi(K) may be rewritten)
     uint64_t *segdone = dsdone + 1;    // the run's dS^T is complete
     uint64_t *dsfree = segdone + 1;    // the drain warps have read the run's dS^T
-    uint64_t *mmadone = dsfree + 1;
-    const int n_bars = 17;             // wfull .. mmadone
+    uint64_t *dzready = dsfree + 1;    // [2] kShort: the token sums of an even / odd run are in shared memory
+    uint64_t *mmadone = dzready + 2;
+    const int n_bars = 19;             // wfull .. mmadone
     uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(bars + n_bars);
     volatile int *fail = reinterpret_cast<volatile int *>(tmem_holder + 1);
 
@@ -239,6 +240,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_prefill(const __grid_constant__
         mbar_init(&ukfree[0], 8);
         mbar_init(&ukfree[1], 8);
         mbar_init(dsfree, 4);
+        for (int i = 0; i < 2; ++i) mbar_init(&dzready[i], 4);   // kShort: the warps of the first two quarters
         *fail = 0;
         fence_mbar_init();
     }
@@ -262,6 +264,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_prefill(const __grid_constant__
     griddep_wait();
     const uint32_t tmem = *tmem_holder;
     uint8_t *stage = smem + a.off_s;
+    // kShort: token sums of a run per quarter, [run mod 2][quarter][2F], in phi(K)'s rows from 64
+    // on, which no product reads (the sums of the run before last have been taken: phi(K) is
+    // written after the previous run's dS^T, which began after the drain before it)
+    float *dzs = reinterpret_cast<float *>(smem + a.off_p + 64 * 128);
 
     if (warp == 0) {
         // ------------------------------------------------------------- producer
@@ -386,6 +392,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_prefill(const __grid_constant__
             if (!Sg || !p.last) continue;
             if (__any_sync(0xffffffffu, !wait_bar(segdone, s & 1u, fail))) break;
             tc_fence_after();
+            if constexpr (kShort) {
+                // one add per feature, the quarters in order: a unit of one run gets the same bits
+                // from run to run
+                if (__any_sync(0xffffffffu, !wait_bar(&dzready[s & 1], (s >> 1) & 1u, fail))) break;
+                const float *dz = dzs + (s & 1) * 4 * F;
+                for (int f = e; f < 2 * F; f += 128) atomicAdd(Sg + (size_t)2 * F * d + f, dz[f] + dz[2 * F + f]);
+            }
             if (32 * (warp & 3) < d) {
 #pragma unroll 1
                 for (int t = 0; t < NC; ++t) {
@@ -421,7 +434,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_prefill(const __grid_constant__
         const uint32_t lane_off = (uint32_t)(32 * q4) << 16;
         const float sgn = part == 0 ? kLog2e : -kLog2e;
         uint8_t *pkb = smem + a.off_p;
-        uint32_t i = 0;
+        uint32_t i = 0, s = 0;
         // token sums of features part*F + 32*jj + dzf
         float dzacc[4] = {0.f, 0.f, 0.f, 0.f};
         const int dzf = 8 * (lane >> 3) + 2 * (lane & 3) + ((lane >> 2) & 1);
@@ -554,7 +567,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_prefill(const __grid_constant__
                     else if (jj == 2) dzacc[2] += y[0];
                     else dzacc[3] += y[0];
                 }
-            } else {
+            } else if (!kShort || q4 < 2) {
                 // a warp beyond the chunk's tokens writes zero rows (the dS^T products
                 // read whole 16-token groups)
 #pragma unroll 1
@@ -576,10 +589,19 @@ __global__ void __launch_bounds__(kThreads, 1) k_prefill(const __grid_constant__
             }
             ++i;
             if (p.last) {
-                // dz of this run: each quarter's token sums, added into z
+                // dz of this run: each quarter's token sums, added into z (kShort: by the drain warps)
 #pragma unroll
-                for (int jj = 0; jj < 4; ++jj)
-                    if (jj < NCH && !bad) atomicAdd(Sg + (size_t)2 * F * d + part * F + 32 * jj + dzf, dzacc[jj]);
+                for (int jj = 0; jj < 4; ++jj) {
+                    const int f = part * F + 32 * jj + dzf;
+                    if (jj >= NCH || bad) continue;
+                    if (!kShort) atomicAdd(Sg + (size_t)2 * F * d + f, dzacc[jj]);
+                    else if (q4 < 2) dzs[(s & 1) * 4 * F + q4 * 2 * F + f] = dzacc[jj];
+                }
+                if (kShort) {
+                    __syncwarp();
+                    if (lane == 0 && q4 < 2 && !bad) mbar_arrive(&dzready[s & 1]);
+                    ++s;
+                }
                 dzacc[0] = dzacc[1] = dzacc[2] = dzacc[3] = 0.f;
             }
             if (__any_sync(0xffffffffu, bad) && *fail) ok = false;
@@ -606,12 +628,12 @@ bool prefill_supported(const hybrid_cfg &c)
 
 // Which of the two tensor-core kernels folds prompts or blocks of up to `longest` tokens into
 // `units` states.  The token-major kernel, which balances chunks across SMs, is the faster one
-// (alone, us, 4 heads, against k_commit_red: d = F = 64, 40 requests of 32 tokens 8.9 against
-// 11.4, 256 requests 23.5 against 35.5; d = F = 128, 64 tokens, 57 requests 18.5 against 21.9;
-// after four steps of 64 requests, d = F = 128, 72.8 against 74.5 for the whole), except for up
-// to 32 tokens with d = F = 128 where whole waves of units fill most SMs: 112 units 11.8 against
-// 11.2, 152: 13.3 against 12.8, 304: 20.3 against 19.8, 456: 27.6 against 27.3 (but 76: 10.0
-// against 10.8, 1024: 55.6 against 57.4; 8 steps and the commit of 512: 194.8 against 201).
+// (alone, us, against k_commit_red: d = F = 64, 40 requests x 8 heads of 32 tokens 12.0 against
+// 16.2; d = 64, F = 128, 64 x 16 of 32 tokens 32.6 against 40.0; d = F = 128, 32 x 4 of 64 tokens
+// 13.1 against 14.2), except for up to 32 tokens with d = F = 128 where whole waves of units fill
+// most SMs: 112 units 11.8 against 11.2, 152: 13.3 against 12.8, 304: 20.3 against 19.8, 456: 27.6
+// against 27.3 (but 76: 10.0 against 10.8, 1024: 55.6 against 57.4; 8 steps and the commit of 512
+// units: 198.6 against 202.3).
 bool commit_by_prefill(const hybrid_cfg &c, int longest, long long units)
 {
     if (!prefill_supported(c)) return false;

@@ -43,3 +43,21 @@ def test_short_commit(n, Hkv, d, F, T, ragged):
     S, z = pair.gpu_state()
     assert_parity(S, pair.S, torch.bfloat16, "state S", units="state")
     assert_parity(z, pair.z, torch.bfloat16, "state z", units="state")
+
+
+def test_short_commit_repeats_bitwise():
+    """64 tokens per request (two warps' token sums): the same bits from run to run."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2608_06628_gb300 import build
+    build.build()
+    wl = wk.Workload("repeat", torch.bfloat16, 400, 2, 2, 128, 128, 32, 69)
+    K, V = wk.prefix_kv(wl, 75, "cuda", n_tok=64)
+    slabs = []
+    for _ in range(4):
+        pair = Pair(wl, tracked=[0])
+        H.hybrid_commit_block(pair.cfg, K, V, 64, pair.W, pair.ptrs, wl.n_req)
+        H.hybrid_commit_block(pair.cfg, V[:, :40].contiguous(), K[:, :40].contiguous(), 40, pair.W, pair.ptrs, wl.n_req)
+        H.hybrid_check()
+        slabs.append(pair.pool.slab.clone())
+    assert all(torch.equal(s, slabs[0]) for s in slabs)
