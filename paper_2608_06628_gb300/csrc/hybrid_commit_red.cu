@@ -281,6 +281,14 @@ __global__ void __launch_bounds__(kThreads, 1) k_commit_red(const __grid_constan
                         if (!wait_bar(&pkready[ci & 1], (ci >> 1) & 1u, fail)) { ok = false; break; }
                         // the previous unit's dS^T has been staged before it is overwritten
                         if (j == 1 && kp > 0 && !wait_bar(dsfree, (kp - 1) & 1u, fail)) { ok = false; break; }
+                        // V's box runs on into the next request: rows beyond the tokens are zeroed, or
+                        // an infinity or NaN there would give NaN times phi(K) = 0
+                        const int nt = Tu - (j - 1) * kChunk;
+                        if (nt < kChunk) {
+                            uint8_t *vrow = smem + a.off_c + (ci & 1) * a.chunk_stride + atom + nt * 128;
+                            for (int p = 0; p < d / 64; ++p) zero_smem(vrow + p * (kChunk * 128), (kChunk - nt) * 128);
+                            fence_proxy_async_smem();
+                        }
                         tc_fence_after();
                         dst(ci, j == 1);
                     }

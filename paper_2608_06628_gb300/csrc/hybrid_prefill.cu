@@ -341,39 +341,52 @@ __global__ void __launch_bounds__(kThreads, 1) k_prefill(const __grid_constant__
             uint32_t pi = 0;
             ChunkPos pp{};
             UnitCache uc;
-            auto issue_ds = [&]() -> bool {
-                if (!wait_bar(pready, pi & 1u, fail) || !wait_bar(&vfull[pi & 1], (pi >> 1) & 1u, fail)) return false;
-                // the previous run's dS^T has been read before this run overwrites it
-                if (pp.first && sd > 0 && !wait_bar(dsfree, (sd - 1) & 1u, fail)) return false;
-                if (pp.first) ++sd;
-                tc_fence_after();
-                dst(pi, pp.nt, pp.first);
-                mma_commit(dsdone);
-                mma_commit(&vfree[pi & 1]);
-                if (pp.last) mma_commit(segdone);
-                return true;
-            };
-            for (ChunkWalk<A> w(a, lo, hi); w.more() && ok; w.next(a)) {
-                const ChunkPos p = w.pos(a);
-                if (!uc.get(a, p.u)) continue;
-                if (p.first) {
-                    if (!wait_bar(wfull, s & 1u, fail)) { ok = false; break; }
-                    ++s;
+            for (ChunkWalk<A> w(a, lo, hi); ok; w.next(a)) {
+                ChunkPos p{};
+                bool more = w.more();
+                if (more) {
+                    p = w.pos(a);
+                    if (!uc.get(a, p.u)) continue;
+                    if (p.first) {
+                        ok = wait_bar(wfull, s & 1u, fail);
+                        ++s;
+                    }
+                    ok = ok && wait_bar(kfull, i & 1u, fail);
+                    if (i >= 2) ok = ok && wait_bar(&ukfree[i & 1], ((i - 2) >> 1) & 1u, fail);
+                    if (!ok) break;
+                    tc_fence_after();
+                    uk(i);
+                    mma_commit(&ukready[i & 1]);
+                    mma_commit(kfree);
+                    if (p.last) mma_commit(wfree);
                 }
-                if (!wait_bar(kfull, i & 1u, fail)) { ok = false; break; }
-                if (i >= 2 && !wait_bar(&ukfree[i & 1], ((i - 2) >> 1) & 1u, fail)) { ok = false; break; }
-                tc_fence_after();
-                uk(i);
-                mma_commit(&ukready[i & 1]);
-                mma_commit(kfree);
-                if (p.last) mma_commit(wfree);
-                if (pend && !issue_ds()) { ok = false; break; }
+                if (pend) {
+                    if (!wait_bar(pready, pi & 1u, fail) || !wait_bar(&vfull[pi & 1], (pi >> 1) & 1u, fail)) break;
+                    // the previous run's dS^T has been read before this run overwrites it
+                    if (pp.first && sd > 0 && !wait_bar(dsfree, (sd - 1) & 1u, fail)) break;
+                    if (pp.first) ++sd;
+                    // the products read whole 16-token groups of V, and its box runs on into the next
+                    // request: those rows are zeroed, or an infinity or NaN there would give NaN
+                    // times phi(K) = 0
+                    const int tail = -pp.nt & 15;
+                    if (tail != 0) {
+                        uint8_t *vrow = smem + a.off_v + (pi & 1) * 2 * kAtom + pp.nt * 128;
+                        zero_smem(vrow, tail * 128);
+                        zero_smem(vrow + kAtom, tail * 128);
+                        fence_proxy_async_smem();
+                    }
+                    tc_fence_after();
+                    dst(pi, pp.nt, pp.first);
+                    mma_commit(dsdone);
+                    mma_commit(&vfree[pi & 1]);
+                    if (pp.last) mma_commit(segdone);
+                }
+                if (!more) break;
                 pend = true;
                 pi = i;
                 pp = p;
                 ++i;
             }
-            if (ok && pend) issue_ds();
             mma_commit(mmadone);
             mbar_wait(mmadone, 0, kWaitNs);
         }

@@ -99,6 +99,12 @@ __device__ __forceinline__ void tma_prefetch_3d(const void *map, int x, int y, i
                  : "memory");
 }
 
+// Zeros to shared memory, one thread: bytes (a multiple of 8) from p on (8-byte aligned).
+__device__ __forceinline__ void zero_smem(void *p, uint32_t bytes)
+{
+    asm volatile("st.bulk.weak.shared::cta [%0], %1, 0;" ::"r"(smem_u32(p)), "l"((uint64_t)bytes) : "memory");
+}
+
 // ------------------------------------------------------------ async copies
 // 1-D bulk copy global -> shared, completion counted on an mbarrier (bytes).
 __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t bytes, uint64_t *bar)
