@@ -143,7 +143,7 @@ hybrid_status hybrid_block_attn(const hybrid_cfg *cfg, const void *Q, const void
     if (hyb::tc_attn_supported(*cfg))
         return from_cuda(hyb::launch_attn_tc(*cfg, Q, K, V, W, alpha, d_state_ptrs, n_req, O, err, stream));
     // the remaining bf16 shapes: split operands on the tensor cores, whatever the size (16
-    // heads, d = F = 128, B = 24: 12.3 us for 1 request and 25 for 16, against 17.8 and 58 on
+    // heads, d = F = 128, B = 24: 12.9 us for 1 request and 26 for 16, against 17.8 and 58 on
     // the CUDA cores, with the same error; below about 9 us both are the host's launch time)
     if (hyb::attn_split_supported(*cfg))
         return from_cuda(hyb::launch_attn_split(*cfg, Q, K, V, W, alpha, d_state_ptrs, n_req, O, err, stream));

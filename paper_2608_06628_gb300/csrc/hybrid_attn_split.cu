@@ -5,12 +5,13 @@
 // These shapes ran float32 FMA kernels and keep that accuracy: bf16 products (U = Q W and
 // the scores) are exact in float32, and every float32 operand of the other products goes in
 // as a sum of parts,
-//   phi S = phi_h S_h + phi_l S_h + phi_h S_l   tf32 parts x = x_h + x_l, x_h = x cut to 11
-//                                               bits: what is left out is 2^-22 of a term
-//   P V   = P_h V + P_l V                       bf16 parts of e^(s - m), 2^-17
+//   phi S = phi_h S_h + phi_l S_h + phi_h S_l   tf32 parts, x_h = x rounded to 11 bits and
+//                                               x_l the rest, itself cut: 2^-22 of a term
+//   P V   = P_h V + P_m V + P_l V               bf16 parts of e^(s - m), 8 bits each: exact
 // so the result differs from the FMA kernels' by less than its own bf16 rounding (2^-9).
-// The merge weights of a row are known before the readout and are folded into phi and P, so
-// one accumulator D takes both branches and holds the output.
+// Infinities stay what the whole product makes of them, not inf - inf or 0 inf: an infinite
+// state element is all in S_l, which only phi_h multiplies, and the parts of a P > 0 are cut,
+// not rounded, and all positive.
 //
 // A work item is 128 of a unit's G B query rows (row t G + h, whole tokens).  One persistent
 // CTA per SM walks a contiguous range of items; 18 warps:
@@ -21,17 +22,20 @@
 //                item on while the rows are still at this one
 //   warp 16      MMA issuer.  S_h and S_l are neighbours and so are the accumulators D and D2,
 //                so phi_h takes both in one product of N = 2 d: 8 MMAs per tile instead of 12
-//                (F = 256 has no room for D2 and issues 12)
+//                (F = 256 has no room for D2 and issues 12).  D2 takes every low product, so
+//                that their additions round nothing off D
 //   warp 17      TMA of an item's Q, W, K, V and z, the next item's during the readout
 // Tensor Memory: [U (64, 128 or 256 columns) | D | D2 | two buffers of phi_h, phi_l], the
 // scores in the phi buffers' columns until P is written.
 //
-// What bounds it: one item takes 12 us with d = F = 128, 1.2 for its loads, 2.9 from U to P
+// What bounds it: one item takes 12.5 us with d = F = 128, 1.2 for its loads, 3.3 from U to P
 // (chains of Tensor Memory loads, exponentials and row exchanges), 0.65 per tile (tensor pipe
-// 0.45) and 1.3 for the output.  16 : 4 heads, d = F = 128, B = 64: 13.7 us for one request,
-// 27.8 for 32; 20.5 and 196 on the CUDA cores (F = 256: 21.8 and 46, against 31.6 and 328).
-// Relative error against 64 bits 1.66e-3 on both, the rounding of a bf16 output.  Two smaller
-// CTAs per SM with single buffers took 16.8 and 29.7 (F = 256: 26.5 and 56).
+// 0.45) and 1.3 for the output.  16 : 4 heads, d = F = 128, B = 64: 14.4 us for one request,
+// 29.9 for 32; 20.5 and 196 on the CUDA cores (F = 256: 22.6 and 47, against 31.6 and 328).
+// Relative error against 64 bits 1.65751e-3 on both, the rounding of a bf16 output; outputs that
+// are not the nearest bf16 value 0.037 % (F = 256, keys x 8: 0.031) against 0.021 (0.030) on the
+// CUDA cores.  P as two rounded parts took 13.8 and 28.6 us, with 0.25 % and NaN for infinities.
+// Two smaller CTAs per SM with single buffers took 2.4 and 1.9 us more (F = 256: 4.7 and 10).
 #include <atomic>
 
 #include "hybrid_common.cuh"
@@ -70,13 +74,13 @@ struct SplitLayout {
     int nbuf;
 };
 
-// Shared memory: [Q | W | K, then P's two parts][S_h | S_l x nbuf][V][z x 2][statistics]
+// Shared memory: [Q | W | K, then P's three parts][S_h | S_l x nbuf][V][z x 2][statistics]
 // [barriers].  Only F = 256 with B > 112 and d = 128 has no room for a second tile buffer.
 SplitLayout make_split_layout(int d, int F, int Bp)
 {
     SplitLayout L{};
     const uint32_t q = (uint32_t)(d / 64) * 128 * 128, w = (uint32_t)((F + 63) / 64) * d * 128;
-    const uint32_t kv = (uint32_t)(d / 64) * Bp * 128, pbytes = 2u * 128 * Bp * 2;
+    const uint32_t kv = (uint32_t)(d / 64) * Bp * 128, pbytes = 3u * 128 * Bp * 2;
     for (L.nbuf = 2; L.nbuf >= 1; --L.nbuf) {
         uint32_t off = q + w + kv > pbytes ? q + w + kv : pbytes;
         L.off_w = q;
@@ -93,8 +97,34 @@ SplitLayout make_split_layout(int d, int F, int Bp)
     return L;
 }
 
-// x cut to a tf32 value (the low 13 bits dropped), and the rest, itself cut by the MMA
-__device__ __forceinline__ float tf32_hi(float x) { return __uint_as_float(__float_as_uint(x) & 0xFFFFE000u); }
+// x rounded to a tf32 value (cvt.rna.tf32 issues at a fraction of the rate of the two)
+__device__ __forceinline__ float tf32_rna(float x)
+{
+    return __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xFFFFE000u);
+}
+// A positive x cut to a bf16 value.
+__device__ __forceinline__ float bf16_hi(float x) { return __uint_as_float(__float_as_uint(x) & 0xFFFF0000u); }
+// What a part h of x >= 0 leaves of rest, positive where x is (2^-40 x is nothing beside h).
+__device__ __forceinline__ float positive_rest(float rest, float h, float x) { return fmaf(x, 0x1p-40f, rest - h); }
+__device__ __forceinline__ uint32_t bf16_pair(float a, float b)   // of values cut to bf16
+{
+    return __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632);
+}
+
+// A thread's granules (stride apart, n of them) of a state tile's parts with an infinite high part
+// among them: that one becomes 0 and the low part all of the element.
+__device__ __noinline__ void split_infinities(float4 *hi, int low, int stride, int n)
+{
+    for (int j = 0; j < n; ++j) {
+        float *h = reinterpret_cast<float *>(hi + j * stride), *l = reinterpret_cast<float *>(hi + low + j * stride);
+        for (int k = 0; k < 4; ++k)
+            if (fabsf(h[k]) == INFINITY) {
+                // (rounded to an infinity, the element itself is finite)
+                l[k] = isnan(l[k]) ? h[k] : copysignf(3.4e38f, h[k]);
+                h[k] = 0.f;
+            }
+    }
+}
 
 // kTwo (F <= 128): two accumulators
 template <bool kTwo>
@@ -113,7 +143,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_attn_split(const __grid_constan
     uint64_t *ldfull = bars;           // Q, W, K and z have landed
     uint64_t *vfull = bars + 1;
     uint64_t *uready = bars + 2;       // U and the scores are formed
-    uint64_t *pready = bars + 3;       // rows -> issuer A: P is written
+    uint64_t *pready = bars + 3;       // rows -> issuer: P is written
     uint64_t *pvdone = bars + 4;       // P V is complete: Q, W, K, P and V space may be reloaded
     uint64_t *opr = bars + 5;          // [2] rows -> issuer: phi's and the state tile's parts
     uint64_t *rdone = bars + 7;        // [2] a tile's products are complete
@@ -207,13 +237,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_attn_split(const __grid_constan
                 if (!wait_bar(pready, k & 1u, fail) || !wait_bar(vfull, k & 1u, fail)) break;
                 if (k > 0 && !wait_bar(dfree, (k - 1) & 1u, fail)) break;
                 tc_fence_after();
-                // P_h V initialises D, P_l V initialises D2
-                for (int h = 0; h < 2; ++h)
+                // P_h V initialises D, P_m V initialises D2
+                for (int h = 0; h < 3; ++h)
                     for (int kk = 0; kk < Bp / 16; ++kk)
                         mma_bf16_ss(h ? d2col : dcol,
                                     smem_desc(s_u + (uint32_t)h * 128 * Bp * 2 + kk * 256, 128, (Bp / 8) * 128, SWZ_NONE),
                                     smem_desc(s_u + a.off_v + 2 * kk * 1024, Bp * 128, 1024, SWZ_128B), idP,
-                                    kTwo ? kk != 0 : (h | kk) != 0);
+                                    kTwo ? h == 2 || kk != 0 : (h | kk) != 0);
                 mma_commit(pvdone);
                 for (int t = 0; t < NT; ++t, ++T) {
                     const uint32_t b = T & a.lbuf;
@@ -225,7 +255,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_attn_split(const __grid_constan
 #pragma unroll
                     for (int kk = 0; kk < 4; ++kk) {
                         const uint64_t bh = smem_desc(sh_u + 32 * kk, 16, 1024, SWZ_128B);
-                        mma_tf32_ts(dcol, al + 8 * kk, bh, idR, 1);
+                        mma_tf32_ts(d2col, al + 8 * kk, bh, idR, 1);
                         if (kTwo) {
                             mma_tf32_ts(dcol, ah + 8 * kk, bh, idR2, 1);
                         } else {
@@ -269,15 +299,19 @@ __global__ void __launch_bounds__(kThreads, 1) k_attn_split(const __grid_constan
                     const uint32_t b = (T + t) & a.lbuf, use = (T + t) >> a.lbuf;
                     if (use > 0) bad = !wait_bar(&rdone[b], (use - 1) & 1u, fail) || bad;
                     float4 *sh = reinterpret_cast<float4 *>(smem + a.off_s + (size_t)b * (2 * d * 128));
+                    float top = 0.f;
 #pragma unroll
                     for (int j = 0; j < 4; ++j)
                         if (j < NS4) {
                             const float4 x = sreg[q][j];
-                            const float4 h = make_float4(tf32_hi(x.x), tf32_hi(x.y), tf32_hi(x.z), tf32_hi(x.w));
+                            const float4 h = make_float4(tf32_rna(x.x), tf32_rna(x.y), tf32_rna(x.z), tf32_rna(x.w));
                             sh[j * (kTileWarps * 32) + st_tid] = h;
                             sh[d * 8 + j * (kTileWarps * 32) + st_tid] =
                                 make_float4(x.x - h.x, x.y - h.y, x.z - h.z, x.w - h.w);
+                            // (fmaxf passes NaN by; the low part of one is NaN whatever the high part)
+                            top = fmaxf(fmaxf(top, fmaxf(fabsf(h.x), fabsf(h.y))), fmaxf(fabsf(h.z), fabsf(h.w)));
                         }
+                    if (top == INFINITY) split_infinities(sh + st_tid, d * 8, kTileWarps * 32, NS4);
                     if (t + kAhead < NT) load_s(sreg[q], Sg, t + kAhead);
                     fence_proxy_async_smem();
                     __syncwarp();
@@ -387,12 +421,14 @@ __global__ void __launch_bounds__(kThreads, 1) k_attn_split(const __grid_constan
                 auto total = [&](int q) { return X(q, 0) + X(q, 1); };
                 const float isp = 1.f / total(4), isn = 1.f / total(5);
                 const float ld = total(6) * isp + total(7) * isn, l = total(3);
-                // merge_weights with the fast intrinsics (this is on the item's critical path)
+                // the weights of merge_weights without its logarithms: e^t l and ld are the
+                // branches' masses, both divided by the larger of e^t and 1
                 float wsm = 0.f, wl = 0.f;
                 if (valid && ld > 0.f) {
-                    const float x = lw + ms * a.inv_sqrt_d + __logf(l) - __logf(ld);   // log of the branches' ratio
-                    wsm = __fdividef(1.f, l * (1.f + __expf(-x)));
-                    wl = __fdividef(1.f, ld * (1.f + __expf(x)));
+                    const float t = lw + ms * a.inv_sqrt_d, e = expf(-fabsf(t));
+                    const float inv = 1.f / (t > 0.f ? fmaf(ld, e, l) : fmaf(l, e, ld));
+                    wsm = t > 0.f ? inv : e * inv;
+                    wl = t > 0.f ? e * inv : inv;
                 } else if (valid) {
                     wsm = lw == -INFINITY ? __int_as_float(0x7fc00000) : 1.f / l;   // empty prefix
                 }
@@ -403,7 +439,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_attn_split(const __grid_constan
             bad = pair_failed(bad);
             const float wsm = X(0, 0), cp = X(0, 1), cn = X(1, 0);
 
-            // ---- P (times its merge weight) as two bf16 parts, K-major without swizzle (core
+            // ---- P (times its merge weight) as three bf16 parts, K-major without swizzle (core
             // matrices of 8 rows x 16 bytes), over Q, W and K, which the products have read
             {
                 uint8_t *prow = smem + (row >> 3) * (Bp / 8) * 128 + (row & 7) * 16;
@@ -412,20 +448,29 @@ __global__ void __launch_bounds__(kThreads, 1) k_attn_split(const __grid_constan
                     float v[16];
                     tmem_ld16(scol + 16 * c, v);
                     tmem_wait_ld();
-                    uint32_t h[8], l[8];
-#pragma unroll
-                    for (int j = 0; j < 16; j += 2) {
-                        const float p0 = 16 * c + j < B ? ex2(fmaf(v[j], scale_l2, -msl)) * wsm : 0.f;
-                        const float p1 = 16 * c + j + 1 < B ? ex2(fmaf(v[j + 1], scale_l2, -msl)) * wsm : 0.f;
-                        h[j / 2] = pack_bf16x2(p0, p1);
-                        l[j / 2] = pack_bf16x2(p0 - __uint_as_float(h[j / 2] << 16),
-                                               p1 - __uint_as_float(h[j / 2] & 0xFFFF0000u));
-                    }
 #pragma unroll
                     for (int j = 0; j < 2; ++j) {
-                        uint8_t *p = prow + (2 * c + j) * 128;
-                        *reinterpret_cast<uint4 *>(p) = make_uint4(h[4 * j], h[4 * j + 1], h[4 * j + 2], h[4 * j + 3]);
-                        *reinterpret_cast<uint4 *>(p + pstride) = make_uint4(l[4 * j], l[4 * j + 1], l[4 * j + 2], l[4 * j + 3]);
+                        uint32_t q[3][4];
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            float h[2], m[2], l[2];
+#pragma unroll
+                            for (int e = 0; e < 2; ++e) {
+                                const int k = 8 * j + 2 * i + e;
+                                const float p = 16 * c + k < B ? ex2(fmaf(v[k], scale_l2, -msl)) * wsm : 0.f;
+                                h[e] = bf16_hi(p);
+                                const float rest = positive_rest(p, h[e], p);
+                                m[e] = bf16_hi(rest);
+                                l[e] = positive_rest(rest, m[e], rest);
+                            }
+                            q[0][i] = bf16_pair(h[0], h[1]);
+                            q[1][i] = bf16_pair(m[0], m[1]);
+                            q[2][i] = bf16_pair(l[0], l[1]);
+                        }
+#pragma unroll
+                        for (int e = 0; e < 3; ++e)
+                            *reinterpret_cast<uint4 *>(prow + e * pstride + (2 * c + j) * 128) =
+                                make_uint4(q[e][0], q[e][1], q[e][2], q[e][3]);
                     }
                 }
             }
@@ -449,7 +494,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_attn_split(const __grid_constan
 #pragma unroll
                     for (int j = 0; j < 16; ++j) {
                         const float x = neg ? ex2(fmaf(-v[j], kLog2e, mnl)) * cn : ex2(fmaf(v[j], kLog2e, -mxl)) * cp;
-                        v[j] = tf32_hi(x);
+                        v[j] = tf32_rna(x);
                         l[j] = x - v[j];
                     }
                 }
