@@ -66,7 +66,8 @@
  * step's other bfloat16 shapes run there too when G divides 128, with every
  * float32 operand as a sum of parts: a probability as three bf16 ones (all of
  * its 24 bits), phi and S as two tf32 ones (2^-22 of a term).  The rest run
- * float32 FMA kernels.
+ * float32 FMA kernels.  An infinity or NaN in V or a state reaches the elements
+ * it reaches in float32, and no other request.
  *
  * Errors: argument checks run synchronously on the host and return
  * HYBRID_ERR_INVALID_ARG (null or misaligned pointer, inconsistent sizes) or

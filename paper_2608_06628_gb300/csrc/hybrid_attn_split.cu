@@ -102,15 +102,6 @@ __device__ __forceinline__ float tf32_rna(float x)
 {
     return __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xFFFFE000u);
 }
-// A positive x cut to a bf16 value.
-__device__ __forceinline__ float bf16_hi(float x) { return __uint_as_float(__float_as_uint(x) & 0xFFFF0000u); }
-// What a part h of x >= 0 leaves of rest, positive where x is (2^-40 x is nothing beside h).
-__device__ __forceinline__ float positive_rest(float rest, float h, float x) { return fmaf(x, 0x1p-40f, rest - h); }
-__device__ __forceinline__ uint32_t bf16_pair(float a, float b)   // of values cut to bf16
-{
-    return __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632);
-}
-
 // A thread's granules (stride apart, n of them) of a state tile's parts with an infinite high part
 // among them: that one becomes 0 and the low part all of the element.
 __device__ __noinline__ void split_infinities(float4 *hi, int low, int stride, int n)

@@ -22,7 +22,11 @@
 // Tensor Memory: [0, 256) U, phi+(q) written over it chunk by chunk; [256, 384) D; [384, 448)
 // phi-(q), two buffers; [448, 512) the scores, then dS^T of a chunk (phi+ | phi- columns).
 // The merge weights of a row are known before the readout and are folded into phi and P (P as
-// two bf16 parts), so D accumulates P V and the readout and is the output.
+// two bf16 parts), so D accumulates P V and the readout and is the output.  The parts are
+// rounded (2^-18), unless V holds an infinity or NaN (the update warps look, while the math warps
+// are at U): a low part that is zero or negative would make NaN of an infinity's product with
+// P, so there the high part is cut and the low one positive (2^-17).  As three cut parts, always,
+// the 256 requests below took 477 us.
 //
 // A ring slot holds one state tile (d rows x 128 bytes) or one 64-column panel of W.  W's four
 // slots and the 16 tiles take 20 items of a 10-slot ring, so W always lands in slots 0-3, in
@@ -126,16 +130,18 @@ __global__ void __launch_bounds__(kThreads, 1) k_fused_wide(const __grid_constan
     uint64_t *vfull = qkfull + 1;
     uint64_t *uready = vfull + 1;      // U and the scores are formed
     uint64_t *pready = uready + 1;     // math -> issuer: P is written
-    uint64_t *dsready = pready + 1;    // dS^T of a chunk is formed
+    uint64_t *vscan = pready + 1;      // update -> math: vbad tells whether V is finite
+    uint64_t *dsready = vscan + 1;     // dS^T of a chunk is formed
     uint64_t *dsfree = dsready + 1;    // update -> issuer: dS^T has been read
     uint64_t *tready = dsfree + 1;     // [kChunks] update -> storer: a chunk's tiles are updated
     uint64_t *udone = tready + kChunks;   // every product of the unit is complete (D; Q, K and V space)
     uint64_t *dfree = udone + 1;       // math -> issuer: D has been read
     uint64_t *zdone = dfree + 1;       // math -> storer: z is updated
     uint64_t *mmadone = zdone + 1;
-    constexpr int n_bars = 2 * NS + 8 + kChunks + 11;
+    constexpr int n_bars = 2 * NS + 8 + kChunks + 12;
     uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(bars + n_bars);
     volatile int *fail = reinterpret_cast<volatile int *>(tmem_holder + 1);
+    int *vbad = reinterpret_cast<int *>(tmem_holder + 2);   // [4] an infinity or NaN in an update warp's part of V
 
     if (tid == 64) {
         prefetch_tensormap(&a.tmQ);
@@ -147,6 +153,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_fused_wide(const __grid_constan
         for (int i = 0; i < n_bars; ++i) mbar_init(&bars[i], 1);
         for (int i = 0; i < 2; ++i) mbar_init(&phi[i], 8);
         mbar_init(pready, 8);
+        mbar_init(vscan, 4);
         mbar_init(dsfree, 4);
         for (int i = 0; i < kChunks; ++i) mbar_init(&tready[i], 4);
         mbar_init(dfree, 4);     // the query warps
@@ -352,9 +359,25 @@ __global__ void __launch_bounds__(kThreads, 1) k_fused_wide(const __grid_constan
         // --------------------------------------------------------------- update
         const int e = 32 * (warp & 3) + lane;
         const uint32_t dscol = tmem + cS + ((uint32_t)(32 * (warp & 3)) << 16);
+        uint32_t k = 0;
         for (int u = u_begin; u < u_end && !*fail; ++u) {
             if (!wide_state(a, u)) continue;
-            bool bad = false;
+            bool bad = !wait_bar(vfull, k & 1u, fail);
+            ++k;
+            {
+                // (0x7f80 + 0x80 reaches the sign's place: an exponent of all ones)
+                uint32_t seen = 0;
+                for (int i = e; i < (d / 64) * kRows * 8; i += 128) {
+                    const uint4 x = reinterpret_cast<const uint4 *>(smem + a.off_v)[i];
+                    seen |= ((x.x & 0x7F807F80u) + 0x00800080u) | ((x.y & 0x7F807F80u) + 0x00800080u) |
+                            ((x.z & 0x7F807F80u) + 0x00800080u) | ((x.w & 0x7F807F80u) + 0x00800080u);
+                }
+                const bool any = __any_sync(0xffffffffu, (seen & 0x80008000u) != 0);
+                if (lane == 0) {
+                    vbad[warp & 3] = any;
+                    if (!bad) mbar_arrive(vscan);
+                }
+            }
             for (int c = 0; c < kChunks; ++c) {
                 bad = !wait_bar(dsready, (uint32_t)c & 1u, fail) || bad;
                 tc_fence_after();
@@ -519,6 +542,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_fused_wide(const __grid_constan
                 if (valid) mw = merge_weights(log_sigmoid(alpha_row), ms * a.inv_sqrt_d, X(7, 0) + X(7, 1), ld);
                 cp *= mw.wl;
                 cn *= mw.wl;
+                bad = !wait_bar(vscan, k & 1u, fail) || bad;
+                const bool finite = (vbad[0] | vbad[1] | vbad[2] | vbad[3]) == 0;
                 uint8_t *prow = xs + (row >> 3) * (kRows / 8) * 128 + (row & 7) * 16;
 #pragma unroll
                 for (int c = 0; c < 2; ++c) {
@@ -531,9 +556,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_fused_wide(const __grid_constan
                         const int j = 32 * part + 16 * c + i;
                         const float p0 = j < B ? ex2(fmaf(v[i], scale_l2, -msl)) * mw.ws : 0.f;
                         const float p1 = j + 1 < B ? ex2(fmaf(v[i + 1], scale_l2, -msl)) * mw.ws : 0.f;
-                        h[i / 2] = pack_bf16x2(p0, p1);
-                        lo[i / 2] = pack_bf16x2(p0 - __uint_as_float(h[i / 2] << 16),
-                                                p1 - __uint_as_float(h[i / 2] & 0xFFFF0000u));
+                        h[i / 2] = finite ? pack_bf16x2(p0, p1) : bf16_pair(p0, p1);
+                        const float h0 = __uint_as_float(h[i / 2] << 16), h1 = __uint_as_float(h[i / 2] & 0xFFFF0000u);
+                        lo[i / 2] = finite ? pack_bf16x2(p0 - h0, p1 - h1)
+                                           : pack_bf16x2(positive_rest(p0, h0, p0), positive_rest(p1, h1, p1));
                     }
 #pragma unroll
                     for (int j = 0; j < 2; ++j) {

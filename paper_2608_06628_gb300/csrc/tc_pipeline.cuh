@@ -34,6 +34,15 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b)
     return *reinterpret_cast<const uint32_t *>(&v);
 }
 
+// Parts of a value x >= 0 as bf16 operands: x cut to a bf16 value; what a part h leaves of rest,
+// positive where x is (2^-40 x is nothing beside h); two values cut to bf16, as one word.
+__device__ __forceinline__ float bf16_hi(float x) { return __uint_as_float(__float_as_uint(x) & 0xFFFF0000u); }
+__device__ __forceinline__ float positive_rest(float rest, float h, float x) { return fmaf(x, 0x1p-40f, rest - h); }
+__device__ __forceinline__ uint32_t bf16_pair(float a, float b)
+{
+    return __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632);
+}
+
 // Bounded wait that also gives up as soon as another role has failed (limit in
 // nanoseconds of %globaltimer; kernels may take it from their arguments).
 __device__ __forceinline__ bool wait_bar(uint64_t *bar, uint32_t parity, volatile int *fail,

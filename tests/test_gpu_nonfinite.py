@@ -22,10 +22,12 @@ def agree(got, want, dt, what, units):
     assert_parity(np.where(fin, got, 0.0), np.where(fin, want, 0.0), dt, what, units=units)
 
 
-# (dtype, n, Hq, Hkv, d, F, B): the split-operand step, its F = 256 form, one state tile; the
-# CUDA cores
+# (dtype, n, Hq, Hkv, d, F, B): the split-operand step, its F = 256 form, one state tile; step
+# and commit at F = 256; the streaming kernels; the CUDA cores
 @pytest.mark.parametrize("dt,n,Hq,Hkv,d,F,B", [
     (BF16, 2, 4, 1, 128, 128, 64), (BF16, 3, 2, 2, 128, 64, 24), (BF16, 2, 8, 1, 64, 256, 40), (BF16, 2, 2, 2, 64, 16, 20),
+    (BF16, 2, 2, 2, 128, 256, 64), (BF16, 3, 8, 2, 64, 256, 16), (BF16, 3, 4, 1, 128, 128, 32), (BF16, 2, 2, 2, 64, 64, 16),
+    (BF16, 2, 2, 1, 128, 128, 48),
     (F32, 2, 4, 2, 64, 64, 17), (BF16, 2, 6, 2, 128, 128, 48),
 ])
 @pytest.mark.parametrize("where", ["values", "state"])
