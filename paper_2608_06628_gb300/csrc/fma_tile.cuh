@@ -181,17 +181,19 @@ struct Staged {
     }
     __device__ __forceinline__ void store_cols(float *tile, int n_cols) const
     {
-const int kq = threadIdx.x & 7, nq = threadIdx.x >> 3;
+        const int kq = threadIdx.x & 7, nq = threadIdx.x >> 3;
         if (4 * nq >= n_cols) return;
         store_block(tile, kq, nq, r);
     }
-    // A state tile (n_rows rows of 128 bytes), already in the tile layout.
+    // A state tile (n_rows rows of 128 bytes), already in the tile layout.  (Plain loads, as for z:
+    // the kernel may start while the one in front still writes the state, so the state is not
+    // read-only for its lifetime, as __ldg asks.)
     __device__ __forceinline__ void load_tile(const float *src, int n_rows)
     {
 #pragma unroll
         for (int q = 0; q < R4; ++q) {
             const int p = threadIdx.x + q * kThreads;
-            if (p < n_rows * 8) r[q] = __ldg(reinterpret_cast<const float4 *>(src) + p);
+            if (p < n_rows * 8) r[q] = reinterpret_cast<const float4 *>(src)[p];
         }
     }
     __device__ __forceinline__ void store_tile(float *tile, int n_rows) const
@@ -290,8 +292,8 @@ __device__ __forceinline__ void phi_rows(const Map<PN, RT> &m, int F, float (&u)
 #pragma unroll
             for (int c = 0; c < CPL; ++c) {
                 const int f = p * PN + m.col(c);
-                zp[p][c] = f < F ? __ldg(z + f) : 0.f;
-                zn[p][c] = f < F ? __ldg(z + F + f) : 0.f;
+                zp[p][c] = f < F ? z[f] : 0.f;
+                zn[p][c] = f < F ? z[F + f] : 0.f;
             }
     }
     float sp[RPL], sn[RPL], lp[RPL], ln[RPL];

@@ -266,13 +266,15 @@ __global__ void __launch_bounds__(kThreads, 1) k_attn_split(const __grid_constan
     } else if (warp >= kRowWarps) {
         // ------------------------------------------------------- state tiles
         const int st_tid = tid - kRowWarps * 32, NS4 = d * 8 / (kTileWarps * 32);
-        // kAhead tiles on their way: a load takes longer than a tile's products
+        // kAhead tiles on their way: a load takes longer than a tile's products.  (Plain loads: the
+        // state may be a running kernel's output when this one starts, so it is not read-only
+        // for the kernel's lifetime, as __ldg asks)
         float4 sreg[kAhead][4];
         auto load_s = [&](float4 (&x)[4], const float *Sg, int t) {
 #pragma unroll
             for (int i = 0; i < 4; ++i)
                 if (i < NS4)
-                    x[i] = __ldg(reinterpret_cast<const float4 *>(Sg) + (size_t)t * 8 * d + i * (kTileWarps * 32) + st_tid);
+                    x[i] = reinterpret_cast<const float4 *>(Sg)[(size_t)t * 8 * d + i * (kTileWarps * 32) + st_tid];
         };
         uint32_t T = 0;
         bool bad = false;
