@@ -406,13 +406,21 @@ __global__ void __launch_bounds__(kThreads, 1) k_commit_red(const __grid_constan
                 const int gf = (f & 63) >> 3;
 #pragma unroll
                 for (int t = 0; t < 32; ++t) {
-                    const float v = ek[t] * __shfl_sync(0xffffffffu, inv_l, t);
-                    dz += v;
-                    if (fval) *reinterpret_cast<bf16 *>(bf + t * 128 + ((gf ^ (t & 7)) << 4)) = __float2bfloat16_rn(v);
+                    ek[t] *= __shfl_sync(0xffffffffu, inv_l, t);
+                    if (fval) *reinterpret_cast<bf16 *>(bf + t * 128 + ((gf ^ (t & 7)) << 4)) = __float2bfloat16_rn(ek[t]);
                 }
                 fence_proxy_async_smem();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&pkready[b]);
+                // the chunk's token sum in the order of k_prefill's warps (tokens 8 apart, then
+                // halves), so that z has the same bits from either kernel
+#pragma unroll
+                for (int t = 0; t < 8; ++t) ek[t] = (ek[t] + ek[t + 8]) + (ek[t + 16] + ek[t + 24]);
+#pragma unroll
+                for (int w = 4; w >= 1; w >>= 1)
+#pragma unroll
+                    for (int t = 0; t < w; ++t) ek[t] += ek[t + w];
+                dz += ek[0];
             }
             if (!ok) break;
             // dz of this thread's feature, then the dS^T tiles into the staging ring

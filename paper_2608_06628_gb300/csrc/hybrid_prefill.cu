@@ -195,7 +195,8 @@ struct ChunkWalk {
 
 // kShort: commits of at most a block's 64 tokens form phi as k_commit_red does (the normaliser
 // added in halves of 32 features, phi = e^(..) / l), which committed them before and still does
-// where it is faster: the bf16 phi(K), and so the state, is the same from either kernel.
+// where it is faster, and both add the 32 tokens of a warp or chunk in the same order to z: a
+// request's state has the same bits whatever batch, and so kernel, it is committed with.
 template <class A, bool kShort>
 __global__ void __launch_bounds__(kThreads, 1) k_prefill(const __grid_constant__ A a)
 {

@@ -70,8 +70,8 @@ cudaError_t launch_phi_tc(const void *X, int n_rows, int nh, int Hkv, int d, int
 // [tok[n_req]][Hkv][d]; tok is a host array read at launch (its values travel in
 // the kernel parameters), so at most kMaxRaggedRequests requests per launch.
 constexpr int kMaxRaggedRequests = 2048;
-// Commits of at most this many tokens per request form phi(K) alike in the block-commit and the
-// prefill kernel (same bits).
+// Commits of at most this many tokens per request form phi(K) and its token sums alike in the
+// block-commit and the prefill kernel (a state of the same bits).
 constexpr int kShortCommit = 64;
 cudaError_t launch_prefill_ragged(const hybrid_cfg &c, const void *K, const void *V, const int *tok, const void *W,
                                   void *const *states, int n_req, unsigned *err, cudaStream_t st);
