@@ -67,7 +67,9 @@
  * float32 operand as a sum of parts: a probability as three bf16 ones (all of
  * its 24 bits), phi and S as two tf32 ones (2^-22 of a term).  The rest run
  * float32 FMA kernels.  An infinity or NaN in V or a state reaches the elements
- * it reaches in float32, and no other request.
+ * it reaches in float32, and no other request.  The same inputs give the same
+ * bits on every call, but for bfloat16 prompts of more than 128 tokens with F in
+ * {64, 128}: their increments are added to the states in any order.
  *
  * Errors: argument checks run synchronously on the host and return
  * HYBRID_ERR_INVALID_ARG (null or misaligned pointer, inconsistent sizes) or

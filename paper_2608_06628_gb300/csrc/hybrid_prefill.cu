@@ -53,6 +53,7 @@ constexpr int kWarps = 16;
 constexpr int kThreads = kWarps * 32;
 constexpr int kCT = 128;             // tokens per chunk (the M of U_k = K W)
 constexpr int kStage = 2;            // staging slots for dS^T tiles
+constexpr uint32_t kHalf = 16 * 128; // kOne: three slots of 16 rows to a drain warp, and dz in the space left
 constexpr int kSmemLimit = 232448;
 constexpr int kOneCtaPerSm = 118 * 1024;
 constexpr uint32_t kColDS = 256;      // dS^T: phi+ features at [256, 256 + F), phi- at [256 + F, 256 + 2F)
@@ -118,7 +119,8 @@ PLayout make_playout(int d, int F)
     L.off_k = off; off += 2 * kAtom;
     L.off_v = off; off += 2 * 2 * kAtom;
     L.off_p = off; off += (uint32_t)(2 * F / 64) * kAtom;
-    L.off_s = off; off += kStage * (uint32_t)d * 128;
+    const uint32_t slots = kStage * (uint32_t)d * 128, halves = (uint32_t)(d / 32) * 3 * kHalf + 2 * 4 * 2 * (uint32_t)F * 4;
+    L.off_s = off; off += slots > halves ? slots : halves;
     L.off_bar = off; off += 1024;
     L.bytes = off + 1024;
     if ((int)L.bytes < kOneCtaPerSm) L.bytes = kOneCtaPerSm;
@@ -197,7 +199,13 @@ struct ChunkWalk {
 // added in halves of 32 features, phi = e^(..) / l), which committed them before and still does
 // where it is faster, and both add the 32 tokens of a warp or chunk in the same order to z: a
 // request's state has the same bits whatever batch, and so kernel, it is committed with.
-template <class A, bool kShort>
+// kOne: longer ones of at most a chunk's 128 tokens.  Both hand the token sums to the drain warps,
+// which add them into z in the quarters' order: a unit is one run, so its state has the same
+// bits from run to run.  In longer prompts the math warps' four quarters add into z as they
+// come, and the runs of a prompt split over CTAs into S: in order, the quarters of 64 prompts of
+// 1 to 4096 tokens took 101 us (waiting for each other) or 108 (kOne's way) against 95.  (64 of 1
+// to 128: 20.4 us against 19.9, at 4 heads; 24 with the adds of one thread per run.)
+template <class A, bool kShort, bool kOne>
 __global__ void __launch_bounds__(kThreads, 1) k_prefill(const __grid_constant__ A a)
 {
     using namespace ptx;
@@ -224,7 +232,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_prefill(const __grid_constant__
     uint64_t *dsdone = pready + 1;     // the chunk's dS^T products are complete (phi(K) may be rewritten)
     uint64_t *segdone = dsdone + 1;    // the run's dS^T is complete
     uint64_t *dsfree = segdone + 1;    // the drain warps have read the run's dS^T
-    uint64_t *dzready = dsfree + 1;    // [2] kShort: the token sums of an even / odd run are in shared memory
+    uint64_t *dzready = dsfree + 1;    // [2] kShort, kOne: the token sums of an even / odd run are in shared memory
     uint64_t *mmadone = dzready + 2;
     const int n_bars = 19;             // wfull .. mmadone
     uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(bars + n_bars);
@@ -241,7 +249,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_prefill(const __grid_constant__
         mbar_init(&ukfree[0], 8);
         mbar_init(&ukfree[1], 8);
         mbar_init(dsfree, 4);
-        for (int i = 0; i < 2; ++i) mbar_init(&dzready[i], 4);   // kShort: the warps of the first two quarters
+        for (int i = 0; i < 2; ++i) mbar_init(&dzready[i], kShort ? 4 : 8);   // the warps of the quarters with tokens
         *fail = 0;
         fence_mbar_init();
     }
@@ -265,10 +273,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_prefill(const __grid_constant__
     griddep_wait();
     const uint32_t tmem = *tmem_holder;
     uint8_t *stage = smem + a.off_s;
-    // kShort: token sums of a run per quarter, [run mod 2][quarter][2F], in phi(K)'s rows from 64
-    // on, which no product reads (the sums of the run before last have been taken: phi(K) is
-    // written after the previous run's dS^T, which began after the drain before it)
-    float *dzs = reinterpret_cast<float *>(smem + a.off_p + 64 * 128);
+    // kShort, kOne: token sums of a run per quarter, [run mod 2][quarter][2F]; kShort: in phi(K)'s
+    // rows from 64 on, which no product reads (the sums of the run before last have been taken:
+    // phi(K) is written after the previous run's dS^T, which began after the drain before it)
+    constexpr int kQuarters = kShort ? 2 : 4;   // with tokens
+    float *dzs = reinterpret_cast<float *>(kShort ? smem + a.off_p + 64 * 128 : smem + a.off_s + (d / 32) * 3 * kHalf);
 
     if (warp == 0) {
         // ------------------------------------------------------------- producer
@@ -395,10 +404,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_prefill(const __grid_constant__
         // ------------------------------------------------------------ drain
         // a run's dS^T out of Tensor Memory and into the state, beside the next run's chunks.
         // A warp owns the 32 rows (e) of its lane quarter: 4 KB of each tile, staged in
-        // two slots of its own, so nothing here waits for another warp
+        // two slots of its own (kOne: three of 16 rows), so nothing here waits for another warp
         const int e = 32 * (warp & 3) + lane;
         const uint32_t lane_off = (uint32_t)(32 * (warp & 3)) << 16;
-        uint32_t s = 0;
+        uint32_t s = 0, half = 0;
         UnitCache uc;
         for (ChunkWalk<A> w(a, lo, hi); w.more(); w.next(a)) {
             const ChunkPos p = w.pos(a);
@@ -406,12 +415,15 @@ __global__ void __launch_bounds__(kThreads, 1) k_prefill(const __grid_constant__
             if (!Sg || !p.last) continue;
             if (__any_sync(0xffffffffu, !wait_bar(segdone, s & 1u, fail))) break;
             tc_fence_after();
-            if constexpr (kShort) {
-                // one add per feature, the quarters in order: a unit of one run gets the same bits
-                // from run to run
+            if constexpr (kShort || kOne) {
+                // one add per feature, the quarters in order
                 if (__any_sync(0xffffffffu, !wait_bar(&dzready[s & 1], (s >> 1) & 1u, fail))) break;
-                const float *dz = dzs + (s & 1) * 4 * F;
-                for (int f = e; f < 2 * F; f += 128) atomicAdd(Sg + (size_t)2 * F * d + f, dz[f] + dz[2 * F + f]);
+                const float *dz = dzs + (s & 1) * kQuarters * 2 * F;
+                for (int f = e; f < 2 * F; f += 128) {
+                    float sum = dz[f] + dz[2 * F + f];
+                    if (kOne) sum += dz[4 * F + f] + dz[6 * F + f];
+                    atomicAdd(Sg + (size_t)2 * F * d + f, sum);
+                }
             }
             if (32 * (warp & 3) < d) {
 #pragma unroll 1
@@ -419,6 +431,26 @@ __global__ void __launch_bounds__(kThreads, 1) k_prefill(const __grid_constant__
                     float v[32];
                     tmem_ld32(tmem + kColDS + lane_off + 32 * t, v);
                     tmem_wait_ld();
+                    if constexpr (kOne) {
+#pragma unroll
+                        for (int h = 0; h < 2; ++h, half = half == 2 ? 0 : half + 1) {
+                            if (lane == 0) bulk_wait_read_2();
+                            __syncwarp();
+                            uint8_t *slot = stage + ((warp & 3) * 3 + half) * kHalf;
+                            if (lane >> 4 == h)
+#pragma unroll
+                                for (int gq = 0; gq < 8; ++gq)
+                                    *reinterpret_cast<float4 *>(slot + (e & 15) * 128 + ((gq ^ (e & 7)) << 4)) =
+                                        make_float4(v[4 * gq], v[4 * gq + 1], v[4 * gq + 2], v[4 * gq + 3]);
+                            fence_proxy_async_smem();
+                            __syncwarp();
+                            if (lane == 0) {
+                                bulk_reduce_add_f32(Sg + (size_t)t * 32 * d + (e + 16 * h) * 32, slot, kHalf);
+                                bulk_commit();
+                            }
+                        }
+                        continue;
+                    }
                     if (lane == 0) bulk_wait_read_1();
                     __syncwarp();
                     uint8_t *rowp = stage + (size_t)(t & 1) * tile + e * 128;
@@ -603,17 +635,17 @@ __global__ void __launch_bounds__(kThreads, 1) k_prefill(const __grid_constant__
             }
             ++i;
             if (p.last) {
-                // dz of this run: each quarter's token sums, added into z (kShort: by the drain warps)
+                // dz of this run: each quarter's token sums, added into z (kShort, kOne: by the drain warps)
 #pragma unroll
                 for (int jj = 0; jj < 4; ++jj) {
                     const int f = part * F + 32 * jj + dzf;
                     if (jj >= NCH || bad) continue;
-                    if (!kShort) atomicAdd(Sg + (size_t)2 * F * d + f, dzacc[jj]);
-                    else if (q4 < 2) dzs[(s & 1) * 4 * F + q4 * 2 * F + f] = dzacc[jj];
+                    if (!kShort && !kOne) atomicAdd(Sg + (size_t)2 * F * d + f, dzacc[jj]);
+                    else if (q4 < kQuarters) dzs[((s & 1) * kQuarters + q4) * 2 * F + f] = dzacc[jj];
                 }
-                if (kShort) {
+                if (kShort || kOne) {
                     __syncwarp();
-                    if (lane == 0 && q4 < 2 && !bad) mbar_arrive(&dzready[s & 1]);
+                    if (lane == 0 && q4 < kQuarters && !bad) mbar_arrive(&dzready[s & 1]);
                     ++s;
                 }
                 dzacc[0] = dzacc[1] = dzacc[2] = dzacc[3] = 0.f;
@@ -690,8 +722,8 @@ bool fill_prefill_args(const hybrid_cfg &c, const void *K, const void *V, long l
     return true;
 }
 
-template <class A, bool kShort>
-cudaError_t run_prefill(const hybrid_cfg &c, const A &a, long long total, cudaStream_t st)
+template <class A, bool kShort, bool kOne>
+cudaError_t run_prefill_as(const hybrid_cfg &c, const A &a, long long total, cudaStream_t st)
 {
     if (total <= 0) return cudaSuccess;
     const PLayout L = make_playout(c.head_dim, c.feat_dim);
@@ -702,7 +734,7 @@ cudaError_t run_prefill(const hybrid_cfg &c, const A &a, long long total, cudaSt
     const unsigned long long bit = 1ull << dev;
     if (!(opted.load(std::memory_order_acquire) & bit)) {
         const cudaError_t e =
-            cudaFuncSetAttribute(k_prefill<A, kShort>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
+            cudaFuncSetAttribute(k_prefill<A, kShort, kOne>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
         if (e != cudaSuccess) return e;
         opted.fetch_or(bit, std::memory_order_acq_rel);
     }
@@ -716,7 +748,14 @@ cudaError_t run_prefill(const hybrid_cfg &c, const A &a, long long total, cudaSt
     at[0].val.programmaticStreamSerializationAllowed = 1;
     lc.attrs = at;
     lc.numAttrs = 1;
-    return cudaLaunchKernelEx(&lc, k_prefill<A, kShort>, a);
+    return cudaLaunchKernelEx(&lc, k_prefill<A, kShort, kOne>, a);
+}
+
+template <class A>
+cudaError_t run_prefill(const hybrid_cfg &c, const A &a, int longest, long long total, cudaStream_t st)
+{
+    if (longest <= kShortCommit) return run_prefill_as<A, true, false>(c, a, total, st);
+    return longest <= kCT ? run_prefill_as<A, false, true>(c, a, total, st) : run_prefill_as<A, false, false>(c, a, total, st);
 }
 
 }  // namespace
@@ -729,8 +768,7 @@ cudaError_t launch_prefill(const hybrid_cfg &c, const void *K, const void *V, in
     a.T = n_tok;
     a.n_chunks = (n_tok + kCT - 1) / kCT;
     const long long total = (long long)a.n_units * a.n_chunks;
-    return n_tok <= kShortCommit ? run_prefill<PrefillArgs, true>(c, a, total, st)
-                                 : run_prefill<PrefillArgs, false>(c, a, total, st);
+    return run_prefill(c, a, n_tok, total, st);
 }
 
 cudaError_t launch_prefill_ragged(const hybrid_cfg &c, const void *K, const void *V, const int *tok, const void *W,
@@ -749,8 +787,7 @@ cudaError_t launch_prefill_ragged(const hybrid_cfg &c, const void *K, const void
     int longest = 0;
     for (int r = 0; r < n_req; ++r) longest = tok[r + 1] - tok[r] > longest ? tok[r + 1] - tok[r] : longest;
     const long long total = (long long)c.n_kv_heads * a.ch[n_req];
-    return longest <= kShortCommit ? run_prefill<PrefillRaggedArgs, true>(c, a, total, st)
-                                   : run_prefill<PrefillRaggedArgs, false>(c, a, total, st);
+    return run_prefill(c, a, longest, total, st);
 }
 
 }  // namespace hyb

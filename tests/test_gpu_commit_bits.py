@@ -1,4 +1,5 @@
-"""The state of a short commit is the same bits from whichever kernel folds it."""
+"""The state of a short commit is the same bits from whichever kernel folds it, and the bits of
+a one-chunk prompt are the same from run to run."""
 import pytest
 import torch
 
@@ -38,3 +39,18 @@ def test_batch_size_does_not_change_a_state(T):
         slabs.append(pair.pool.slab.clone())
     for s in slabs[1:]:
         assert torch.equal(s, slabs[0])
+
+
+@pytest.mark.parametrize("d,F", [(128, 128), (64, 128), (128, 64), (64, 64)])
+def test_one_chunk_prompt_repeats_bitwise(d, F):
+    """65 to 128 tokens per request (four warps' token sums): the same bits from run to run."""
+    wl = wk.Workload("repeat", torch.bfloat16, 400, 2, 2, d, F, 32, 94)
+    K, V = wk.prefix_kv(wl, 75, "cuda", n_tok=128)
+    slabs = []
+    for _ in range(6):
+        pair = Pair(wl, tracked=[0])
+        for T in (128, 100, 70):
+            H.hybrid_commit_block(pair.cfg, K[:, :T].contiguous(), V[:, :T].contiguous(), T, pair.W, pair.ptrs, wl.n_req)
+        H.hybrid_check()
+        slabs.append(pair.pool.slab.clone())
+    assert all(torch.equal(s, slabs[0]) for s in slabs)
