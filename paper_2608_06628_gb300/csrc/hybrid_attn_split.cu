@@ -152,10 +152,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_attn_split(const __grid_constan
         prefetch_tensormap(&a.tmW);
         prefetch_tensormap(&a.tmK);
         prefetch_tensormap(&a.tmV);
-        for (int i = 0; i < n_bars; ++i) mbar_init(&bars[i], 1);
-        mbar_init(pready, kRowWarps);
-        mbar_init(dfree, kRowWarps);
-        for (int i = 0; i < 2; ++i) mbar_init(&opr[i], kRowWarps + kTileWarps);
+        mbar_init_n(ldfull, 3, 1);   // vfull, uready
+        mbar_init_n(pready, 1, kRowWarps);
+        mbar_init_n(pvdone, 1, 1);
+        mbar_init_n(opr, 2, kRowWarps + kTileWarps);
+        mbar_init_n(rdone, 3, 1);    // ddone
+        mbar_init_n(dfree, 1, kRowWarps);
+        mbar_init_n(mmadone, 1, 1);
         *fail = 0;
         fence_mbar_init();
     }

@@ -153,14 +153,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_commit_red(const __grid_constan
         prefetch_tensormap(&a.tmW);
     }
     if (tid == 0) {
-        for (int i = 0; i < n_bars; ++i) mbar_init(&bars[i], 1);
-        for (int b = 0; b < 2; ++b) {
-            mbar_init(&cfull[b], 2);
-            mbar_init(&pkready[b], 8);
-        }
-        for (int s = 0; s < kStage; ++s) mbar_init(&sfull[s], 4);   // the four warps of one part
-        mbar_init(dsfree, 8);
-        mbar_init(dzready, 8);
+        mbar_init_n(cfull, 2, 2);
+        mbar_init_n(cfree, 4, 1);             // ukready
+        mbar_init_n(pkready, 2, 8);
+        mbar_init_n(sfull, kStage, 4);        // the four warps of one part
+        mbar_init_n(sempty, kStage + 3, 1);   // wfull, wfree, dsready
+        mbar_init_n(dsfree, 2, 8);            // dzready
+        mbar_init_n(dzfree, 2, 1);            // mmadone
         *fail = 0;
         fence_mbar_init();
     }

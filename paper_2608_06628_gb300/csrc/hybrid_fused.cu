@@ -216,16 +216,17 @@ __global__ void __launch_bounds__(kThreads, 1) k_fused(const __grid_constant__ F
     }
     if (warp == 3 && lane == 0) prefetch_tensormap(&a.tmO);
     if (tid == 0) {
-        for (int i = 0; i < n_bars; ++i) mbar_init(&bars[i], 1);
-        mbar_init(xfull, 2);
-        mbar_init(phip, 8);
-        mbar_init(phim, 8);
-        mbar_init(pready, 8);
-        for (int i = 0; i < 2; ++i) mbar_init(&tready[i], 8);
-        mbar_init(kready, 8);
-        mbar_init(efree, 8);
-        mbar_init(zdone, 8);
-        mbar_init(ostaged, 8);
+        mbar_init_n(full, 2 * NS + 6, 1);   // empty, zfull, zempty, dready
+        mbar_init_n(tready, 2, 8);
+        mbar_init_n(xfull, 1, 2);
+        mbar_init_n(uready, 1, 1);
+        mbar_init_n(phip, 3, 8);            // phim, pready
+        mbar_init_n(mmadone, 3, 1);         // xfree, vfull
+        mbar_init_n(kready, 1, 8);
+        mbar_init_n(dsdone, 2, 1);          // pvdone
+        mbar_init_n(efree, 2, 8);           // zdone
+        mbar_init_n(ofree, 1, 1);
+        mbar_init_n(ostaged, 1, 8);
         *fail = 0;
         fence_mbar_init();
     }

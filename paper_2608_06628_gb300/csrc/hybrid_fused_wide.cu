@@ -150,14 +150,16 @@ __global__ void __launch_bounds__(kThreads, 1) k_fused_wide(const __grid_constan
         prefetch_tensormap(&a.tmW);
     }
     if (tid == 0) {
-        for (int i = 0; i < n_bars; ++i) mbar_init(&bars[i], 1);
-        for (int i = 0; i < 2; ++i) mbar_init(&phi[i], 8);
-        mbar_init(pready, 8);
-        mbar_init(vscan, 4);
-        mbar_init(dsfree, 4);
-        for (int i = 0; i < kChunks; ++i) mbar_init(&tready[i], 4);
-        mbar_init(dfree, 4);     // the query warps
-        mbar_init(zdone, 4);     // the key warps
+        mbar_init_n(full, 2 * NS + 4, 1);     // empty, zfull, zempty
+        mbar_init_n(phi, 2, 8);
+        mbar_init_n(rdone, 6, 1);             // wfull, qkfull, vfull, uready
+        mbar_init_n(pready, 1, 8);
+        mbar_init_n(vscan, 1, 4);
+        mbar_init_n(dsready, 1, 1);
+        mbar_init_n(dsfree, 1 + kChunks, 4);  // tready
+        mbar_init_n(udone, 1, 1);
+        mbar_init_n(dfree, 2, 4);             // the query warps; zdone: the key warps
+        mbar_init_n(mmadone, 1, 1);
         *fail = 0;
         fence_mbar_init();
     }

@@ -77,9 +77,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_phi_tc(const __grid_constant__ 
     if (tid == 0) {
         prefetch_tensormap(&a.tmX);
         prefetch_tensormap(&a.tmW);
-        for (int i = 0; i < 7; ++i) mbar_init(&bars[i], 1);
-        mbar_init(&ufree[0], kWarps);
-        mbar_init(&ufree[1], kWarps);
+        mbar_init_n(xfull, 4, 1);   // ufull
+        mbar_init_n(ufree, 2, kWarps);
+        mbar_init_n(wfull, 1, 1);
         *fail = 0;
         fence_mbar_init();
     }

@@ -244,12 +244,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_prefill(const __grid_constant__
         prefetch_tensormap(&a.tmW);
     }
     if (tid == 0) {
-        for (int i = 0; i < n_bars; ++i) mbar_init(&bars[i], 1);
-        mbar_init(pready, 8);
-        mbar_init(&ukfree[0], 8);
-        mbar_init(&ukfree[1], 8);
-        mbar_init(dsfree, 4);
-        for (int i = 0; i < 2; ++i) mbar_init(&dzready[i], kShort ? 4 : 8);   // the warps of the quarters with tokens
+        mbar_init_n(wfull, 10, 1);                 // wfree, kfull, kfree, vfull, vfree, ukready
+        mbar_init_n(ukfree, 3, 8);                 // pready
+        mbar_init_n(dsdone, 2, 1);                 // segdone
+        mbar_init_n(dsfree, 1, 4);
+        mbar_init_n(dzready, 2, kShort ? 4 : 8);   // the warps of the quarters with tokens
+        mbar_init_n(mmadone, 1, 1);
         *fail = 0;
         fence_mbar_init();
     }

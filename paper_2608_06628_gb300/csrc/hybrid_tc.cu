@@ -195,9 +195,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_attn_tc(const __grid_constant__
     int *issued = fail + 1;   // S chunks of the unit issued so far (for draining after a failure)
 
     if (tid == 0) {
-        for (int i = 0; i < 2 * RM + 7; ++i) mbar_init(&bars[i], 1);
-        mbar_init(bar_d, 2);
-        mbar_init(bar_p, 2);
+        mbar_init_n(bars, 2 * RM + 2, 1);   // full, empty, bar_z, bar_u
+        mbar_init_n(bar_d, 2, 2);           // bar_p
+        mbar_init_n(bar_u2, 3, 1);          // bar_ld, bar_b
         *fail = 0;
         fence_mbar_init();
     }

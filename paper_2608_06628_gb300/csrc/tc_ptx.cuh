@@ -26,6 +26,11 @@ __device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count)
 {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
 }
+// n neighbouring barriers (each barrier of a kernel is initialised once)
+__device__ __forceinline__ void mbar_init_n(uint64_t *bars, int n, uint32_t count)
+{
+    for (int i = 0; i < n; ++i) mbar_init(bars + i, count);
+}
 __device__ __forceinline__ void fence_mbar_init()
 {
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
