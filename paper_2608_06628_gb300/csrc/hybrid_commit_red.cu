@@ -479,7 +479,8 @@ bool commit_red_supported(const hybrid_cfg &c)
 {
     if (c.io_dtype != HYBRID_BF16) return false;
     if (c.head_dim != 64 && c.head_dim != 128) return false;
-    if (c.feat_dim != 64 && c.feat_dim != 128 && c.feat_dim != 256) return false;
+    // (k_prefill takes every commit with a smaller d F)
+    if (c.feat_dim != 256 && (c.feat_dim != 128 || c.head_dim != 128)) return false;
     return (int)make_clayout(c.head_dim, c.feat_dim).bytes <= kSmemLimit;
 }
 

@@ -46,31 +46,9 @@ __host__ __device__ __forceinline__ size_t z_offset(int f, int d, int F)
     return (size_t)2 * F * d + f;
 }
 
-// For granule p (16 bytes) of tile `tile` (d rows x 8 granules, in storage
-// order): the row e and the first logical feature f of the 4 floats it holds.
-__host__ __device__ __forceinline__ void granule_coords(int p_in_tile, int tile, int &e, int &f0)
-{
-    e = p_in_tile >> 3;
-    const int j = (p_in_tile & 7) ^ (e & 7);
-    f0 = tile * 32 + 4 * j;
-}
-
 __device__ __forceinline__ bool state_ptr_ok(const void *p)
 {
     return p != nullptr && (reinterpret_cast<uintptr_t>(p) & 15u) == 0;
-}
-
-// ---------------------------------------------------------------------------
-// io dtype loads / stores
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ float to_f32(float x) { return x; }
-__device__ __forceinline__ float to_f32(__nv_bfloat16 x) { return __bfloat162float(x); }
-
-template <typename T> __device__ __forceinline__ T from_f32(float x);
-template <> __device__ __forceinline__ float from_f32<float>(float x) { return x; }
-template <> __device__ __forceinline__ __nv_bfloat16 from_f32<__nv_bfloat16>(float x)
-{
-    return __float2bfloat16_rn(x);
 }
 
 __device__ __forceinline__ float warp_max(float v)

@@ -39,7 +39,7 @@ struct PhiTcArgs {
     float *Phi;
     unsigned *err;
     long long rows;         // (row, head) pairs per state head
-    int n_tiles, tiles_per_g, nh, log_group, d, F;
+    int n_tiles, tiles_per_g, nh, log_group, d;
 };
 
 template <int F>
@@ -319,7 +319,6 @@ cudaError_t launch_phi_tc(const void *X, int n_rows, int nh, int Hkv, int d, int
     a.log_group = 0;
     while ((1 << a.log_group) < group) ++a.log_group;
     a.d = d;
-    a.F = F;
     if (F == 64) return launch_phi<64>(a, st);
     if (F == 128) return launch_phi<128>(a, st);
     return launch_phi<256>(a, st);

@@ -683,7 +683,7 @@ bool prefill_supported(const hybrid_cfg &c)
 bool commit_by_prefill(const hybrid_cfg &c, int longest, long long units)
 {
     if (!prefill_supported(c)) return false;
-    if (!commit_red_supported(c) || longest > 32 || c.head_dim < 128 || c.feat_dim < 128) return true;
+    if (!commit_red_supported(c) || longest > 32) return true;
     const int sms = sm_count();
     return 2 * units <= sms || units > 3ll * sms;
 }

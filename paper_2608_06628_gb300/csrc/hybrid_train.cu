@@ -94,8 +94,6 @@ __device__ __forceinline__ uint32_t swz(int r, int j)
     return (uint32_t)r * 128u + (uint32_t)((j ^ (r & 7)) << 4);
 }
 
-__device__ __forceinline__ void bulk_wait_read_1() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
-
 // Write kN consecutive columns [c0, c0 + kN) of row r (values x, converted to
 // bf16) into a bf16 operand image with panel stride pstride.
 template <int kN>
