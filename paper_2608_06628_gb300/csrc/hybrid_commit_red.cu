@@ -25,6 +25,7 @@
 // the math warps' two parts on the two feature tiles instead of the two signs,
 // and dS^T of the pass's sign in [256,512).
 #include <atomic>
+#include <type_traits>
 
 #include "hybrid_common.cuh"
 #include "hybrid_tc.h"
@@ -47,8 +48,8 @@ constexpr int kOneCtaPerSm = 118 * 1024;
 constexpr uint32_t kColDSp = 256, kColDSm = 384;
 
 struct CommitArgs {
-    CUtensorMap tmV, tmW;   // V [n*T][Hkv][d], W [Hkv*d][F]; 128-byte swizzle, 64-element panels
-                            // as the outermost box dimension (one copy for all of them)
+    CUtensorMap tmV, tmW;   // V [n][T][Hkv][d] (ragged: [tokens][Hkv][d]), W [Hkv*d][F]; 128-byte swizzle,
+                            // 64-element panels as the outermost box dimension (one copy for all of them)
     CUtensorMap tmK;        // K as V (used only to prefetch K into L2; K is read by the warps)
     const bf16 *K;
     void *const *states;
@@ -92,6 +93,32 @@ struct CommitRaggedArgs : CommitArgs {
     int n_req;
     int tok[kMaxRaggedRequests + 1];
 };
+// A chunk's V rows, into shared memory or L2 only (K too).  Its products read all 32 of them, and
+// phi(K) is zero beyond the tokens, but an infinity or NaN there would make NaN of it: uniform
+// boxes are filled with zeros beyond the request's tokens; ragged ones run on into the next
+// request, and the issuer zeroes those rows.
+__device__ __forceinline__ void load_v(const CommitArgs &a, void *dst, int u, int j, uint64_t *bar)
+{
+    const int hu = u / a.n_pass;
+    ptx::tma_load_5d(dst, &a.tmV, 0, hu % a.Hkv, j * kChunk, hu / a.Hkv, 0, bar);
+}
+__device__ __forceinline__ void load_v(const CommitRaggedArgs &a, void *dst, int u, int j, uint64_t *bar)
+{
+    const int hu = u / a.n_pass;
+    ptx::tma_load_4d(dst, &a.tmV, 0, hu % a.Hkv, a.tok[hu / a.Hkv] + j * kChunk, 0, bar);
+}
+__device__ __forceinline__ void prefetch_kv(const CommitArgs &a, int u, int j)
+{
+    const int hu = u / a.n_pass;
+    ptx::tma_prefetch_5d(&a.tmK, 0, hu % a.Hkv, j * kChunk, hu / a.Hkv, 0);
+    ptx::tma_prefetch_5d(&a.tmV, 0, hu % a.Hkv, j * kChunk, hu / a.Hkv, 0);
+}
+__device__ __forceinline__ void prefetch_kv(const CommitRaggedArgs &a, int u, int j)
+{
+    const int hu = u / a.n_pass;
+    ptx::tma_prefetch_4d(&a.tmK, 0, hu % a.Hkv, a.tok[hu / a.Hkv] + j * kChunk, 0);
+    ptx::tma_prefetch_4d(&a.tmV, 0, hu % a.Hkv, a.tok[hu / a.Hkv] + j * kChunk, 0);
+}
 // tokens of unit u and the K/V row of its first token, uniform or ragged
 __device__ __forceinline__ int unit_len(const CommitArgs &a, int) { return a.T; }
 __device__ __forceinline__ long long unit_tok0(const CommitArgs &a, int u)
@@ -113,15 +140,17 @@ __device__ __forceinline__ float *unit_head(const CommitArgs &a, int u)
     return st + (size_t)(hu % a.Hkv) * head_floats(a.d, a.F);
 }
 
-template <class A>
+// kWide: F = 256, one sign per pass
+template <class A, bool kWide>
 __global__ void __launch_bounds__(kThreads, 1) k_commit_red(const __grid_constant__ A a)
 {
     using namespace ptx;
+    constexpr bool kRagged = std::is_same_v<A, CommitRaggedArgs>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int d = a.d, F = a.F;
-    const bool wide = a.n_pass > 1;       // F = 256: one sign per pass
+    constexpr bool wide = kWide;
     const int NH = F / 32;                 // dS^T tiles per half
     const int NCP = wide ? NH : 2 * NH;    // dS^T tiles per pass
     const uint32_t atom = (uint32_t)d * 128;
@@ -174,12 +203,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_commit_red(const __grid_constan
     // drains: a prefetch brings no value into the SM, so it needs no ordering after it
     if (tid == 64)
         for (int u = u_begin; u < u_end && u < u_begin + 2; ++u) {
-            const int Tu = unit_len(a, u), g = (u / a.n_pass) % a.Hkv;
-            const int tok0 = (int)unit_tok0(a, u);
-            for (int j = 0; j * kChunk < Tu && j < 2; ++j) {
-                tma_prefetch_4d(&a.tmK, 0, g, tok0 + j * kChunk, 0);
-                tma_prefetch_4d(&a.tmV, 0, g, tok0 + j * kChunk, 0);
-            }
+            const int Tu = unit_len(a, u);
+            for (int j = 0; j * kChunk < Tu && j < 2; ++j) prefetch_kv(a, u, j);
         }
     griddep_wait();
     const uint32_t tmem = *tmem_holder;
@@ -214,7 +239,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_commit_red(const __grid_constan
                 if (__any_sync(0xffffffffu, !ok)) break;
                 if (lane == 0) {
                     mbar_arrive_expect_tx(&cfull[b], vbytes);
-                    tma_load_4d(cb + atom, &a.tmV, 0, g, (int)tok0 + j * kChunk, 0, &cfull[b]);
+                    load_v(a, cb + atom, u, j, &cfull[b]);
                 }
                 ++nv;
                 kt_store(kr, d, cb, lane);
@@ -280,13 +305,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_commit_red(const __grid_constan
                         if (!wait_bar(&pkready[ci & 1], (ci >> 1) & 1u, fail)) { ok = false; break; }
                         // the previous unit's dS^T has been staged before it is overwritten
                         if (j == 1 && kp > 0 && !wait_bar(dsfree, (kp - 1) & 1u, fail)) { ok = false; break; }
-                        // V's box runs on into the next request: rows beyond the tokens are zeroed, or
-                        // an infinity or NaN there would give NaN times phi(K) = 0
-                        const int nt = Tu - (j - 1) * kChunk;
-                        if (nt < kChunk) {
-                            uint8_t *vrow = smem + a.off_c + (ci & 1) * a.chunk_stride + atom + nt * 128;
-                            for (int p = 0; p < d / 64; ++p) zero_smem(vrow + p * (kChunk * 128), (kChunk - nt) * 128);
-                            fence_proxy_async_smem();
+                        if constexpr (kRagged) {
+                            const int nt = Tu - (j - 1) * kChunk;
+                            if (nt < kChunk) {
+                                uint8_t *vrow = smem + a.off_c + (ci & 1) * a.chunk_stride + atom + nt * 128;
+                                for (int p = 0; p < d / 64; ++p) zero_smem(vrow + p * (kChunk * 128), (kChunk - nt) * 128);
+                                fence_proxy_async_smem();
+                            }
                         }
                         tc_fence_after();
                         dst(ci, j == 1);
@@ -406,20 +431,23 @@ __global__ void __launch_bounds__(kThreads, 1) k_commit_red(const __grid_constan
 #pragma unroll
                 for (int t = 0; t < 32; ++t) {
                     ek[t] *= __shfl_sync(0xffffffffu, inv_l, t);
+                    if (kWide) dz += ek[t];
                     if (fval) *reinterpret_cast<bf16 *>(bf + t * 128 + ((gf ^ (t & 7)) << 4)) = __float2bfloat16_rn(ek[t]);
                 }
                 fence_proxy_async_smem();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&pkready[b]);
-                // the chunk's token sum in the order of k_prefill's warps (tokens 8 apart, then
-                // halves), so that z has the same bits from either kernel
+                if constexpr (!kWide) {
+                    // the chunk's token sum in the order of k_prefill's warps (tokens 8 apart, then
+                    // halves), so that z has the same bits from either kernel
 #pragma unroll
-                for (int t = 0; t < 8; ++t) ek[t] = (ek[t] + ek[t + 8]) + (ek[t + 16] + ek[t + 24]);
+                    for (int t = 0; t < 8; ++t) ek[t] = (ek[t] + ek[t + 8]) + (ek[t + 16] + ek[t + 24]);
 #pragma unroll
-                for (int w = 4; w >= 1; w >>= 1)
+                    for (int w = 4; w >= 1; w >>= 1)
 #pragma unroll
-                    for (int t = 0; t < w; ++t) ek[t] += ek[t + w];
-                dz += ek[0];
+                        for (int t = 0; t < w; ++t) ek[t] += ek[t + w];
+                    dz += ek[0];
+                }
             }
             if (!ok) break;
             // dz of this thread's feature, then the dS^T tiles into the staging ring
@@ -486,20 +514,24 @@ bool commit_red_supported(const hybrid_cfg &c)
 
 namespace {
 
-// Tensor maps and sizes shared by the uniform and the ragged launch; rows = tokens of K and V.
-bool fill_commit_args(const hybrid_cfg &c, const void *K, const void *V, long long rows, const void *W,
+// Tensor maps and sizes shared by the uniform and the ragged launch: K and V of `rows` tokens
+// (T = 0) or of n_req requests with T tokens each.
+bool fill_commit_args(const hybrid_cfg &c, const void *K, const void *V, long long rows, int T, const void *W,
                       void *const *states, int n_req, unsigned *err, CommitArgs &a)
 {
     const CLayout L = make_clayout(c.head_dim, c.feat_dim);
     const int d = c.head_dim, F = c.feat_dim, Hkv = c.n_kv_heads;
-    // V: [panel][row][head][64], a box of kChunk rows of one head; W: [panel][row][64]
-    const cuuint64_t dv[4] = {64, (cuuint64_t)Hkv, (cuuint64_t)rows, (cuuint64_t)d / 64};
-    const cuuint64_t sv[3] = {(cuuint64_t)d * 2, (cuuint64_t)Hkv * d * 2, 128};
-    const cuuint32_t bv[4] = {64, 1, (cuuint32_t)kChunk, (cuuint32_t)d / 64};
+    // V: [panel][row][head][64] or [panel][request][row][head][64], a box of kChunk rows of one
+    // head; W: [panel][row][64]
+    const int rank = T > 0 ? 5 : 4;
+    const cuuint64_t P = (cuuint64_t)d / 64, row = (cuuint64_t)Hkv * d * 2;
+    const cuuint64_t dv[5] = {64, (cuuint64_t)Hkv, (cuuint64_t)(T > 0 ? T : rows), T > 0 ? (cuuint64_t)n_req : P, P};
+    const cuuint64_t sv[4] = {(cuuint64_t)d * 2, row, T > 0 ? row * T : 128, 128};
+    const cuuint32_t bv[5] = {64, 1, (cuuint32_t)kChunk, T > 0 ? 1u : (cuuint32_t)P, (cuuint32_t)P};
     const cuuint64_t dw[3] = {64, (cuuint64_t)Hkv * d, (cuuint64_t)F / 64};
     const cuuint64_t sw[2] = {(cuuint64_t)F * 2, 128};
     const cuuint32_t bw[3] = {64, (cuuint32_t)d, (cuuint32_t)F / 64};
-    if (!encode_bf16(&a.tmV, V, 4, dv, sv, bv) || !encode_bf16(&a.tmK, K, 4, dv, sv, bv) ||
+    if (!encode_bf16(&a.tmV, V, rank, dv, sv, bv) || !encode_bf16(&a.tmK, K, rank, dv, sv, bv) ||
         !encode_bf16(&a.tmW, W, 3, dw, sw, bw))
         return false;
     a.K = static_cast<const bf16 *>(K);
@@ -520,8 +552,8 @@ bool fill_commit_args(const hybrid_cfg &c, const void *K, const void *V, long lo
     return true;
 }
 
-template <class A>
-cudaError_t run_commit_red(const hybrid_cfg &c, const A &a, cudaStream_t st)
+template <class A, bool kWide>
+cudaError_t run_commit_red_as(const hybrid_cfg &c, const A &a, cudaStream_t st)
 {
     const CLayout L = make_clayout(c.head_dim, c.feat_dim);
     const int grid = a.n_units < sm_count() ? a.n_units : sm_count();
@@ -531,7 +563,7 @@ cudaError_t run_commit_red(const hybrid_cfg &c, const A &a, cudaStream_t st)
     const unsigned long long bit = 1ull << dev;
     if (!(opted.load(std::memory_order_acquire) & bit)) {
         const cudaError_t e =
-            cudaFuncSetAttribute(k_commit_red<A>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
+            cudaFuncSetAttribute(k_commit_red<A, kWide>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
         if (e != cudaSuccess) return e;
         opted.fetch_or(bit, std::memory_order_release);
     }
@@ -545,7 +577,13 @@ cudaError_t run_commit_red(const hybrid_cfg &c, const A &a, cudaStream_t st)
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     lc.attrs = attr;
     lc.numAttrs = 1;
-    return cudaLaunchKernelEx(&lc, k_commit_red<A>, a);
+    return cudaLaunchKernelEx(&lc, k_commit_red<A, kWide>, a);
+}
+
+template <class A>
+cudaError_t run_commit_red(const hybrid_cfg &c, const A &a, cudaStream_t st)
+{
+    return a.n_pass > 1 ? run_commit_red_as<A, true>(c, a, st) : run_commit_red_as<A, false>(c, a, st);
 }
 
 }  // namespace
@@ -554,7 +592,7 @@ cudaError_t launch_commit_red(const hybrid_cfg &c, const void *K, const void *V,
                               void *const *states, int n_req, unsigned *err, cudaStream_t st)
 {
     CommitArgs a;
-    if (!fill_commit_args(c, K, V, (long long)n_req * n_tok, W, states, n_req, err, a)) return cudaErrorInvalidValue;
+    if (!fill_commit_args(c, K, V, 0, n_tok, W, states, n_req, err, a)) return cudaErrorInvalidValue;
     a.T = n_tok;
     return run_commit_red(c, a, st);
 }
@@ -564,7 +602,7 @@ cudaError_t launch_commit_red_ragged(const hybrid_cfg &c, const void *K, const v
 {
     if (n_req < 1 || n_req > kMaxRaggedRequests) return cudaErrorInvalidValue;
     static thread_local CommitRaggedArgs a;   // 8 KB of offsets: kept off the stack
-    if (!fill_commit_args(c, K, V, tok[n_req] > 0 ? tok[n_req] : 1, W, states, n_req, err, a))
+    if (!fill_commit_args(c, K, V, tok[n_req] > 0 ? tok[n_req] : 1, 0, W, states, n_req, err, a))
         return cudaErrorInvalidValue;
     a.T = 0;
     a.n_req = n_req;
