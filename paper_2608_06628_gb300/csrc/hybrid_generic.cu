@@ -39,10 +39,11 @@ int pick_rows(long long units, long long rows, bool allow64)
 // ---------------------------------------------------------------------------
 // Feature map: Phi = [softmax(X W_g), softmax(-X W_g)] for RT rows of the heads of one
 // state head (row i of group g is (i / group, g * group + i % group)), so that W_g is
-// read once per RT rows (float32 rows and F < 64; bf16 rows run in hybrid_phi.cu).  4096
-// rows x 16 heads, d = F = 128: 320 us with one warp per row and head (W_g read from L1 by
-// every warp), 124 us now; the FMA pipes' floor is 28 us, the rest is the staging of X and W
-// and the exponentials, with 8 warps per SM to hide them.
+// read once per RT rows (float32 rows, and bf16 ones with F < 64; the others run in
+// hybrid_phi.cu).  4096 float32 rows x 16 heads, d = F = 128: 329 us with one warp per row and
+// head (W_g read from L1 by every warp), 124 us now (bf16 rows, F = 32: 290 and 84); the FMA
+// pipes' floor is 28 us, the rest is the staging of X and W and the exponentials, with 8 warps
+// per SM to hide them.
 // ---------------------------------------------------------------------------
 struct PhiArgs {
     const void *X, *W;
