@@ -204,7 +204,7 @@ struct ChunkWalk {
 // bits from run to run.  In longer prompts the math warps' four quarters add into z as they
 // come, and the runs of a prompt split over CTAs into S: in order, the quarters of 64 prompts of
 // 1 to 4096 tokens took 101 us (waiting for each other) or 108 (kOne's way) against 95.  (64 of 1
-// to 128: 20.4 us against 19.9, at 4 heads; 24 with the adds of one thread per run.)
+// to 128: 20.3 us against 20.0, at 4 heads; 24 with the adds of one thread per run.)
 template <class A, bool kShort, bool kOne>
 __global__ void __launch_bounds__(kThreads, 1) k_prefill(const __grid_constant__ A a)
 {
@@ -413,10 +413,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_prefill(const __grid_constant__
             const ChunkPos p = w.pos(a);
             float *Sg = uc.get(a, p.u);
             if (!Sg || !p.last) continue;
-            if (__any_sync(0xffffffffu, !wait_bar(segdone, s & 1u, fail))) break;
-            tc_fence_after();
             if constexpr (kShort || kOne) {
-                // one add per feature, the quarters in order
+                // one add per feature, the quarters in order, while the products run (after them, 8
+                // steps and the commit of 512 units took 0.7 us more)
                 if (__any_sync(0xffffffffu, !wait_bar(&dzready[s & 1], (s >> 1) & 1u, fail))) break;
                 const float *dz = dzs + (s & 1) * kQuarters * 2 * F;
                 for (int f = e; f < 2 * F; f += 128) {
@@ -425,6 +424,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_prefill(const __grid_constant__
                     atomicAdd(Sg + (size_t)2 * F * d + f, sum);
                 }
             }
+            if (__any_sync(0xffffffffu, !wait_bar(segdone, s & 1u, fail))) break;
+            tc_fence_after();
             if (32 * (warp & 3) < d) {
 #pragma unroll 1
                 for (int t = 0; t < NC; ++t) {
@@ -432,23 +433,27 @@ __global__ void __launch_bounds__(kThreads, 1) k_prefill(const __grid_constant__
                     tmem_ld32(tmem + kColDS + lane_off + 32 * t, v);
                     tmem_wait_ld();
                     if constexpr (kOne) {
+                        // two of the three half slots: the one before last and, of the tile
+                        // before, the first half's
+                        const uint32_t next = half == 2 ? 0 : half + 1;
+                        uint8_t *slots = stage + (warp & 3) * 3 * kHalf;
+                        if (lane == 0) bulk_wait_read_1();
+                        __syncwarp();
+                        uint8_t *rowp = slots + (lane < 16 ? half : next) * kHalf + (e & 15) * 128;
 #pragma unroll
-                        for (int h = 0; h < 2; ++h, half = half == 2 ? 0 : half + 1) {
-                            if (lane == 0) bulk_wait_read_2();
-                            __syncwarp();
-                            uint8_t *slot = stage + ((warp & 3) * 3 + half) * kHalf;
-                            if (lane >> 4 == h)
-#pragma unroll
-                                for (int gq = 0; gq < 8; ++gq)
-                                    *reinterpret_cast<float4 *>(slot + (e & 15) * 128 + ((gq ^ (e & 7)) << 4)) =
-                                        make_float4(v[4 * gq], v[4 * gq + 1], v[4 * gq + 2], v[4 * gq + 3]);
-                            fence_proxy_async_smem();
-                            __syncwarp();
-                            if (lane == 0) {
-                                bulk_reduce_add_f32(Sg + (size_t)t * 32 * d + (e + 16 * h) * 32, slot, kHalf);
-                                bulk_commit();
-                            }
+                        for (int gq = 0; gq < 8; ++gq)
+                            *reinterpret_cast<float4 *>(rowp + ((gq ^ (e & 7)) << 4)) =
+                                make_float4(v[4 * gq], v[4 * gq + 1], v[4 * gq + 2], v[4 * gq + 3]);
+                        fence_proxy_async_smem();
+                        __syncwarp();
+                        if (lane == 0) {
+                            float *dst = Sg + (size_t)t * 32 * d + e * 32;
+                            bulk_reduce_add_f32(dst, slots + half * kHalf, kHalf);
+                            bulk_commit();
+                            bulk_reduce_add_f32(dst + 16 * 32, slots + next * kHalf, kHalf);
+                            bulk_commit();
                         }
+                        half = next == 2 ? 0 : next + 1;
                         continue;
                     }
                     if (lane == 0) bulk_wait_read_1();
