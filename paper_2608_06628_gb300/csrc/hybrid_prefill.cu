@@ -681,14 +681,14 @@ bool prefill_supported(const hybrid_cfg &c)
 // `units` states.  Above 32 tokens, and with d or F of 64, the token-major kernel, which balances
 // chunks across SMs, is the faster one at every size (alone, us, against k_commit_red: d = F = 64,
 // 40 requests x 8 heads of 32 tokens 12.0 against 16.2; d = 64, F = 128, 64 x 16 of 32 tokens 32.6
-// against 40.0; d = F = 128, 33 to 64 tokens 9.9 against 12.4 for 16 - 76 units, 14 against 15 for
-// 152, 28.5 against 32 - 33 for 456, 57 against 65 - 68 for 1024).
+// against 40.0; d = F = 128, 33 to 64 tokens 9.7 against 12.4 for 16 - 76 units, 11 against 13 for
+// 152, 27.5 against 31 for 456, 56 against 64 - 67 for 1024).
 // Up to 32 tokens with d = F = 128 (us, the other first, k_prefill second):
 //   units                     76    112   152   228   304   380   456   512   608   768   1024
-//   the commit alone       10.2  10.6  12.0  17.8  19.7  26.0  27.4  32.4  34.9  43.5   57.1
-//                           9.8  10.6  12.9  17.7  20.7  25.5  28.3  32.7  35.5  46.3   56.5
-//   four steps and it      42.1  45.8  47.9  72.9  75.9 100.5 107.0 119.1 140.3 165.3  202.4
-//                          41.6  45.4  47.7  72.5  74.0  97.7 103.6 114.1 137.5 161.1  199.3
+//   the commit alone       10.1  10.3  11.5  17.6  19.6  25.6  27.2  32.4  34.9  43.2   57.2
+//                           9.4  10.5  12.6  17.6  20.6  25.0  28.0  32.0  35.1  45.2   56.0
+//   four steps and it      41.8  45.1  47.3  70.9  75.0  98.7 105.4 117.6 139.2 162.2  201.2
+//                          41.0  44.6  47.0  70.8  72.6  96.2 101.8 112.2 136.2 158.0  196.5
 // so k_commit_red keeps commits between half a wave of units and three, where it is ahead by
 // itself in whole waves; from there on the commit of a decode loop, which starts under the last
 // step, decides for the other.
