@@ -198,7 +198,7 @@ struct ChunkWalk {
 // kShort: commits of at most a block's 64 tokens form phi as k_commit_red does (the normaliser
 // added in halves of 32 features, phi = e^(..) / l), which committed them before and still does
 // where it is faster, and both add the 32 tokens of a warp or chunk in the same order to z: a
-// request's state has the same bits whatever batch, and so kernel, it is committed with.
+// request's state has the same bits whatever batch of such commits, and so kernel, it is in.
 // kOne: longer ones of at most a chunk's 128 tokens.  Both hand the token sums to the drain warps,
 // which add them into z in the quarters' order: a unit is one run, so its state has the same
 // bits from run to run.  In longer prompts the math warps' four quarters add into z as they
